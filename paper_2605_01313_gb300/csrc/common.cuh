@@ -176,6 +176,34 @@ __host__ __device__ __forceinline__ int dfs_tpitch(int herm, int N1) {
     return herm ? ((N1 / 2 + 1 + 3) & ~3) : N1;
 }
 
+// The theta-pass output of one line.  16-byte complex values are stored row by
+// row.  FP32 values are stored by pairs of rows (2r, 2r + 1), the unit both
+// FP32 passes transform together (fft_pair.cuh): column q of the pair is the
+// 16 bytes (re, re, im, im) of the two rows, so that the theta pass writes and
+// the phi pass reads both with one access and two neighbouring columns fill a
+// 32-byte sector.
+template <typename C>
+__device__ __forceinline__ void t_store(C *line, int row, int col, int pitch, C v) {
+    if constexpr (sizeof(C) == 8) {
+        float *d = reinterpret_cast<float *>(line) + ((size_t)(row >> 1) * pitch + col) * 4 +
+                   (row & 1);
+        d[0] = v.x;
+        d[2] = v.y;
+    } else {
+        line[(size_t)row * pitch + col] = v;
+    }
+}
+template <typename C>
+__device__ __forceinline__ C t_load(const C *line, int row, int col, int pitch) {
+    if constexpr (sizeof(C) == 8) {
+        const float *d = reinterpret_cast<const float *>(line) +
+                         ((size_t)(row >> 1) * pitch + col) * 4 + (row & 1);
+        return cmake(d[0], d[2]);
+    } else {
+        return line[(size_t)row * pitch + col];
+    }
+}
+
 // Bytes of one unsorted point record of set_points (points.cu FoldRec): packed
 // base cell and rank (two ints) and the two offsets in plan precision.
 __host__ __device__ __forceinline__ int dfs_fold_rec_bytes(int dtype) {
@@ -207,6 +235,10 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
 cudaError_t dfs_launch_theta_pass(dfsnufft_plan p, const void *coeffs, int prM = -1,
                                   int prN = -1);
 cudaError_t dfs_launch_phi_pass(dfsnufft_plan p);
+// The FP32 forms (fft_theta_pair.cu, fft_phi_pair.cu): cudaErrorNotSupported,
+// without launching, for the shapes they do not take.
+cudaError_t dfs_launch_theta_pair(dfsnufft_plan p, const void *coeffs, int prM, int prN);
+cudaError_t dfs_launch_phi_pair(dfsnufft_plan p);
 // Largest FP64 exponent of each of lines line0 .. line0 + lines - 1 into
 // p->d_emax (the double-single scaling of df32.cuh): every one of the
 // line_elems complex values of a line, or (herm) those a real-field theta pass

@@ -11,7 +11,8 @@
 // pass already transformed the Hermitian part of the coefficients, so its row
 // holds H_k itself for k = 0..N1/2, and H_{-k} = conj H_k.  Each CTA handles CB
 // rows inside the plan's needed row range; the row's values are staged in
-// shared memory first, since every one of them enters two Z_k.
+// shared memory first, since every one of them enters two Z_k.  FP32 plans with
+// fine rows of 2^7 to 2^13 cells run k_phi_pair (fft_phi_pair.cu) instead.
 #include <type_traits>
 
 #include "fft_core.cuh"
@@ -53,13 +54,13 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int c = threadIdx.x / T;
     const int row = row0 + c;
     const int f = a.line0 + blockIdx.y;
-    const C *src = in + ((size_t)f * a.n2 + row) * a.tpitch;
+    const C *src = in + (size_t)f * a.n2 * a.tpitch;
     R *dst = grid + ((size_t)f * a.n2 + row) * a.n1;
     const int half = a.N1 / 2;
     const int nmask = a.n1 - 1;
     C *sm = smem + (size_t)c * region_len<C>(M);
     C *srow = smem + (size_t)a.CB * region_len<C>(M) + (size_t)c * a.tcols;
-    for (int i = t; i < a.tcols; i += T) srow[i] = src[i];
+    for (int i = t; i < a.tcols; i += T) srow[i] = t_load(src, row, i, a.tpitch);
     __syncthreads();
     auto hval = [&](int k) -> C {              // real-field rows: H_k, k taken mod n1
         k &= nmask;
@@ -104,79 +105,6 @@ __global__ void __launch_bounds__(MAXT, MINB)
     };
     if constexpr (LOGM > 0) line_fft_ct<LOGM, E>(stw, sm, t, ld, st);
     else line_fft<E>(a.logm, tw, 1, sm, t, ld, st);
-}
-
-// FP32 rows at compile-time lengths: each thread group transforms two rows
-// at once (line_fft_ct2: the twiddles, the index arithmetic and the barriers
-// serve both).  grid (n2 / CB, lines), CB = 2 x threads / (M/E) rows a CTA.
-template <int E, int MAXT, int MINB, int LOGM, bool HERM>
-__global__ void __launch_bounds__(MAXT, MINB)
-    k_phi_pass2(PhiArgs a, const float2 *__restrict__ in, const float2 *__restrict__ tw,
-                const float2 *__restrict__ stw, const int2 *__restrict__ rowrange,
-                float *__restrict__ grid) {
-    dfs_grid_wait();
-    typedef float2 C;
-    const int row0 = blockIdx.x * a.CB;
-    const int2 rr = rowrange[(a.line0 + blockIdx.y) / a.F];
-    if (((row0 - rr.x) & (a.n2 - 1)) >= rr.y) return;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *smem = reinterpret_cast<C *>(smem_raw);
-    constexpr int M = 1 << LOGM;
-    constexpr int T = M / E;
-    const int t = threadIdx.x % T;
-    const int c = threadIdx.x / T;                 // row pair
-    const int row = row0 + 2 * c;
-    const int f = a.line0 + blockIdx.y;
-    const int half = a.N1 / 2;
-    const int nmask = a.n1 - 1;
-    const C *src = in + ((size_t)f * a.n2 + row) * a.tpitch;
-    float *dst = grid + ((size_t)f * a.n2 + row) * a.n1;
-    C *sm0 = smem + (size_t)(2 * c) * region_len<C>(M);
-    C *sm1 = sm0 + region_len<C>(M);
-    C *srow0 = smem + (size_t)a.CB * region_len<C>(M) + (size_t)(2 * c) * a.tcols;
-    C *srow1 = srow0 + a.tcols;
-    for (int i = t; i < a.tcols; i += T) {
-        srow0[i] = src[i];
-        srow1[i] = src[a.tpitch + i];
-    }
-    __syncthreads();
-    // H_k of a row (k mod n1): real-field rows hold H_k, k = 0..N1/2; general
-    // rows hold T_k and H_k = (T_k + conj T_{-k}) / 2
-    auto hval = [&](const C *sr, int k) -> C {
-        k &= nmask;
-        if constexpr (HERM) {
-            if (k <= half) return sr[k];
-            if (k >= a.n1 - half) {
-                const C v = sr[a.n1 - k];
-                return cmake(v.x, -v.y);
-            }
-            return cmake(0.f, 0.f);
-        } else {
-            auto tv = [&](int kk) -> C {
-                kk &= nmask;
-                if (kk < half) return sr[kk + half];
-                if (kk >= a.n1 - half) return sr[kk - a.n1 + half];
-                return cmake(0.f, 0.f);
-            };
-            const C p = tv(k), m = tv(-k);
-            return cmake(0.5f * (p.x + m.x), 0.5f * (p.y - m.y));
-        }
-    };
-    auto ld2 = [&](int k, C &z0, C &z1) {
-        const C w = __ldg(&tw[k]);
-        const C a0 = hval(srow0, k), b0 = hval(srow0, k + M);
-        const C a1 = hval(srow1, k), b1 = hval(srow1, k + M);
-        const C d0 = cmul(cmake(a0.x - b0.x, a0.y - b0.y), w);
-        const C d1 = cmul(cmake(a1.x - b1.x, a1.y - b1.y), w);
-        z0 = cmake(a0.x + b0.x - d0.y, a0.y + b0.y + d0.x);
-        z1 = cmake(a1.x + b1.x - d1.y, a1.y + b1.y + d1.x);
-    };
-    auto st2 = [&](int j, C z0, C z1) {
-        reinterpret_cast<C *>(dst)[j] = z0;
-        reinterpret_cast<C *>(dst + a.n1)[j] = z1;
-    };
-    auto none = [] {};
-    line_fft_ct2<LOGM, E>(stw, sm0, sm1, t, ld2, st2, none);
 }
 
 // Per precision: elements per thread E, threads per CTA at most MAXT with MINB
@@ -226,29 +154,15 @@ cudaError_t dispatch_phi(dfsnufft_plan p, const PhiArgs &a, size_t smem, dim3 gr
     if (threads > MAXT) return run_phi<R, MAXTW, 1, 0, HERM>(p, a, smem, grid, threads);
     // compile-time lengths need the plan's stage-ordered table (double-single
     // for df32)
-    if (std::is_same<R, df32>::value ? !p->d_df_stw_phi : !p->d_stw_phi)
-        return run_phi<R, MAXT, MINB, 0, HERM>(p, a, smem, grid, threads);
-    switch (a.logm) {
-        case 9: return run_phi<R, MAXT, MINB, 9, HERM>(p, a, smem, grid, threads);
-        case 10: return run_phi<R, MAXT, MINB, 10, HERM>(p, a, smem, grid, threads);
-        case 11: return run_phi<R, MAXT, MINB, 11, HERM>(p, a, smem, grid, threads);
-        default: return run_phi<R, MAXT, MINB, 0, HERM>(p, a, smem, grid, threads);
+    if constexpr (!std::is_same<R, float>::value) {
+        switch ((std::is_same<R, df32>::value ? p->d_df_stw_phi : p->d_stw_phi) ? a.logm : 0) {
+            case 9: return run_phi<R, MAXT, MINB, 9, HERM>(p, a, smem, grid, threads);
+            case 10: return run_phi<R, MAXT, MINB, 10, HERM>(p, a, smem, grid, threads);
+            case 11: return run_phi<R, MAXT, MINB, 11, HERM>(p, a, smem, grid, threads);
+            default: break;
+        }
     }
-}
-
-// Four CTAs of 256 threads an SM (at most 64 registers a thread; about 51 KB of
-// shared memory each for rows of 2048): the row loads at the start of each CTA
-// are latency-bound, and the fourth CTA hides more of them than the registers
-// a thread gives up cost (2 us of 64 on the 2048 x 1024 rows).
-template <int LOGM, bool HERM>
-cudaError_t run_phi2(dfsnufft_plan p, const PhiArgs &a, size_t smem, dim3 grid, int threads) {
-    constexpr int E = PhiCfg<float>::E;
-    cudaError_t e = allow_smem(k_phi_pass2<E, 256, 4, LOGM, HERM>, smem);
-    if (e) return e;
-    return dfs_launch_dependent(k_phi_pass2<E, 256, 4, LOGM, HERM>, grid, dim3(threads), smem,
-                                p->stream, a, (const float2 *)p->d_T, (const float2 *)p->d_tw1,
-                                (const float2 *)p->d_stw_phi, (const int2 *)p->d_rowrange,
-                                (float *)p->d_G);
+    return run_phi<R, MAXT, MINB, 0, HERM>(p, a, smem, grid, threads);
 }
 
 template <typename R>
@@ -268,21 +182,6 @@ cudaError_t launch_phi(dfsnufft_plan p) {
     dfs_lines(p, a.line0, lines);
     const int M = q.n1 / 2;
     const int T = M / E;
-    if (sizeof(R) == 4 && p->d_stw_phi && a.logm >= 9 && a.logm <= 11) {
-        // two rows a thread group, 256 threads a CTA
-        a.CB = 2 * (256 / T);
-        const size_t smem = sizeof(C) * (size_t)a.CB * (region_len<C>(M) + a.tcols);
-        const dim3 grid(q.n2 / a.CB, lines);
-        const int threads = (a.CB / 2) * T;
-        switch (a.logm) {
-            case 9: return p->herm ? run_phi2<9, true>(p, a, smem, grid, threads)
-                                   : run_phi2<9, false>(p, a, smem, grid, threads);
-            case 10: return p->herm ? run_phi2<10, true>(p, a, smem, grid, threads)
-                                    : run_phi2<10, false>(p, a, smem, grid, threads);
-            default: return p->herm ? run_phi2<11, true>(p, a, smem, grid, threads)
-                                    : run_phi2<11, false>(p, a, smem, grid, threads);
-        }
-    }
     int cb = MAXT / T;
     if (cb < 1) cb = 1;
     if (cb > DFS_ROW_BLOCK) cb = DFS_ROW_BLOCK;
@@ -299,5 +198,7 @@ cudaError_t launch_phi(dfsnufft_plan p) {
 
 cudaError_t dfs_launch_phi_pass(dfsnufft_plan p) {
     if (p->gdf) return launch_phi<df32>(p);           // FP64 plans in double-single
-    return p->prm.dtype == DFSNUFFT_F64 ? launch_phi<double>(p) : launch_phi<float>(p);
+    if (p->prm.dtype == DFSNUFFT_F64) return launch_phi<double>(p);
+    const cudaError_t e = dfs_launch_phi_pair(p);
+    return e == cudaErrorNotSupported ? launch_phi<float>(p) : e;
 }

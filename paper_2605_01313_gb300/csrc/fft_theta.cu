@@ -17,16 +17,17 @@
 // a general plan.  Column m = 0 takes its Hermitian part in full (its mirror is
 // the same column).  This halves the column transforms and the T buffer.
 //
-// Main kernel (k_theta_tma): persistent CTAs take blocks of CB columns (16- or
-// 32-byte row segments).  The block's N2 coefficient rows arrive in shared memory by
-// 2-D TMA boxes, double-buffered so that the next block streams in while this
-// one is transformed.  Each column's length-n2 transform is done as two
-// length-n2/2 transforms: output row 2q + s = sum_n c_n e^{2 pi i n s / n2}
-// e^{2 pi i n q / (n2/2)}, s = 0, 1 (the modes fit in n2/2; when n2 = 2 N2 the
-// two Nyquist modes n = -N2/2 and n = +N2/2 of a real-field plan share index
-// N2/2 and are added there).  k_theta_pass is the plain-load version for shapes
-// the TMA kernel does not take (unaligned coefficient pointer, CTA or
-// shared-memory limits).
+// FP32 plans run k_theta_pair (fft_theta_pair.cu) at fine sizes of 2^7 to 2^13
+// rows.  k_theta_tma here serves FP64 plans with points in the caller's order:
+// persistent CTAs take blocks of CB columns whose N2 coefficient rows arrive in
+// shared memory by 2-D TMA boxes, double-buffered so that the next block
+// streams in while this one is transformed.  Each column's length-n2 transform
+// is done as two length-n2/2 transforms: output row 2q + s = sum_n c_n
+// e^{2 pi i n s / n2} e^{2 pi i n q / (n2/2)}, s = 0, 1 (the modes fit in n2/2;
+// when n2 = 2 N2 the two Nyquist modes n = -N2/2 and n = +N2/2 of a real-field
+// plan share index N2/2 and are added there).  k_theta_pass is the plain-load
+// version: FP64 plans in double-single arithmetic, and the shapes the other two
+// do not take (unaligned coefficient pointer, CTA or shared-memory limits).
 #include <type_traits>
 
 #include "coef_map.cuh"
@@ -37,58 +38,6 @@ using namespace dfs_fft;
 using namespace dfs_coef;
 
 namespace {
-
-// A coefficient as the pass's complex type: itself, or (double-single passes of
-// FP64 plans) the FP64 value times 2^-sh (the line's exponent shift, df32.cuh)
-// split into double-single parts.
-template <typename C, typename CIn> __device__ __forceinline__ C in_value(CIn v, int) { return v; }
-template <> __device__ __forceinline__ dfc in_value<dfc, double2>(double2 v, int sh) {
-    return to_dfc_scaled(v, sh);
-}
-// Complex coefficient c_{n,m} (m >= 0, |n| <= N) of a field given by its
-// partial-regularity DFS coefficients (Sec. 4): col[k] = f^c_{k,m} + i f^s_{k,m},
-// k = 0..N, for this m.  First the standard coefficient S = f~^c + i f~^s at |n|
-// (the product-to-sum stencil of Sec. 4 for the case of m; f~_{0,m} = f_{1,m}/2
-// for even m >= 2, which the identity gives in place of the printed 0), then
-// Eq. 5.4: c = S/2 (m = 0, n != 0; S for n = 0), conj(S)/2 or /4 (even m), and
-// -sign(n) i conj(S)/4 (odd m).  The stencils are linear with real weights, so
-// they act on the cosine and sine parts at once.
-template <typename C, typename CIn>
-__device__ __forceinline__ C pr_coef(int n, int m, int N, const CIn *__restrict__ col,
-                                     int sh = 0) {
-    typedef decltype(C().x) R;
-    const int na = n < 0 ? -n : n;
-    // f_{k,m} on the case's index range, zero elsewhere
-    auto f = [&](int k, int lo, int hi) -> C {
-        return (k >= lo && k <= hi) ? in_value<C>(col[k], sh) : cmake((R)0, (R)0);
-    };
-    C S;
-    if (m == 0) {
-        if (na > N) return cmake((R)0, (R)0);
-        const R v = in_value<C>(col[na], sh).x;            // no sine part at m = 0
-        return cmake(na == 0 ? v : (R)0.5 * v, (R)0);
-    } else if (m == 1) {
-        if (na == 0) return cmake((R)0, (R)0);
-        // sin t cos k t = (sin (k+1) t - sin (k-1) t) / 2, k = 0..N-1
-        S = cscale(f(na - 1, 0, N - 1) - f(na + 1, 0, N - 1), (R)0.5);
-        if (na == 1) S = S + cscale(f(0, 0, N - 1), (R)0.5);
-    } else if ((m & 1) == 0) {
-        // sin t sin k t = (cos (k-1) t - cos (k+1) t) / 2, k = 1..N-1
-        S = na == 0 ? cscale(f(1, 1, N - 1), (R)0.5)
-                    : cscale(f(na + 1, 1, N - 1) - f(na - 1, 1, N - 1), (R)0.5);
-    } else {
-        if (na == 0) return cmake((R)0, (R)0);
-        // sin^2 t sin k t = (2 sin k t - sin (k-2) t - sin (k+2) t) / 4, k = 1..N-2
-        S = cscale(cscale(f(na, 1, N - 2), (R)2) - f(na - 2, 1, N - 2) - f(na + 2, 1, N - 2),
-                   (R)0.25);
-        if (na == 1) S = S + cscale(f(1, 1, N - 2), (R)0.25);
-    }
-    const C cs = cmake(S.x, -S.y);                         // conj(S) = f~^c - i f~^s
-    if ((m & 1) == 0) return cscale(cs, na == 0 ? (R)0.5 : (R)0.25);
-    // -sign(n) i conj(S) / 4
-    const R g = n > 0 ? (R)-0.25 : (R)0.25;
-    return cmake(-g * cs.y, g * cs.x);
-}
 
 // Largest biased FP64 exponent of each line's coefficients (emax[line], zeroed
 // before the launch; the double-single passes scale the line by it, df32.cuh),
@@ -159,7 +108,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int2 rr = rowrange[f / a.F];
     const bool col_ok = q < a.tcols;
     const CIn *cf0 = coef + (size_t)f * a.N2 * a.N1;
-    C *dst = out + (size_t)f * a.n2 * a.tpitch + q;
+    C *dst = out + (size_t)f * a.n2 * a.tpitch;
     const int half = a.N2 / 2;
     const int qa = HERM ? a.N1 / 2 + q : q;        // array column
     const R sq = col_ok ? inv1[qa < a.N1 ? qa : 0] : (R)0;
@@ -189,7 +138,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
         }
     };
     auto st = [&](int i, C v) {
-        if (col_ok && ((i - rr.x) & (a.n2 - 1)) < rr.y) dst[(size_t)i * a.tpitch] = v;
+        if (col_ok && ((i - rr.x) & (a.n2 - 1)) < rr.y) t_store(dst, i, q, a.tpitch, v);
     };
     if constexpr (LOGN > 0) line_fft_ct<LOGN, E>(stw, sm, t, ld, st);
     else line_fft<E>(a.logn2, tw, 0, sm, t, ld, st);
@@ -210,14 +159,10 @@ struct ThetaTmaArgs {
     int line0;                // first line of the launch (blocks cover lines line0 ..)
 };
 
-// LOGH > 0: half length 2^LOGH fixed at compile time (unrolled transform);
-// LOGH == 0: taken from the arguments.  DUAL (FP32 at compile-time lengths):
-// the two half-length transforms of a column run together in the same threads
-// (line_fft_ct2: twiddles, index arithmetic and barriers shared), which needs
-// one input buffer only: the next block's boxes are issued as soon as every
-// thread has read its inputs (after the transforms' first barrier), so they
-// land while this block is transformed.  Otherwise the halves run one after
-// the other and the next block streams into a second buffer when one fits.
+// FP64 plans with points in the caller's order.  LOGH > 0: half length 2^LOGH
+// fixed at compile time (unrolled transform); LOGH == 0: taken from the
+// arguments.  The two half-length transforms of a column run one after the
+// other and the next block streams into a second buffer when one fits.
 // PRIN (real-field plans): the input is partial-regularity DFS coefficients,
 // lines x (prM + 1) x (prN + 1) complex, whose column m is contiguous; a block's
 // CB columns are staged by 8-byte asynchronous copies of every thread instead of
@@ -233,7 +178,6 @@ __global__ void __launch_bounds__(MAXT, MINB)
                 typename CxT<R>::type *__restrict__ out, int *__restrict__ status) {
     dfs_grid_wait();
     typedef typename CxT<R>::type C;
-    constexpr bool DUAL = LOGH > 0 && sizeof(R) == 4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     // TMA destinations start on 128-byte boundaries (base rounded up here;
     // buffer and box sizes are multiples of 128 bytes by construction)
@@ -242,16 +186,12 @@ __global__ void __launch_bounds__(MAXT, MINB)
     C *inb = reinterpret_cast<C *>(base + 128);
     C *ex = inb + (size_t)a.nbuf * a.in_elems;
     const int H = LOGH ? (1 << LOGH) : (a.n2 >> 1);
-    constexpr int NREG = DUAL ? 2 : 1;             // exchange regions per column
-    R *f2 = reinterpret_cast<R *>(ex + (size_t)NREG * CB * region_len<C>(H));   // 1 / phihat2
+    R *f2 = reinterpret_cast<R *>(ex + (size_t)CB * region_len<C>(H));   // 1 / phihat2
     C *nyq = reinterpret_cast<C *>(f2 + ((a.N2 + 3) & ~3));   // real-field plans: CB values
     const int c = threadIdx.x % CB;
     const int t = threadIdx.x / CB;
     const int half = a.N2 / 2;
-    // column c's regions c and (DUAL: its odd-row transform) CB + c, region_stride
-    // apart (the columns of a warp on different bank pairs)
     C *sm = ex + (size_t)c * region_stride<C>(H, CB);
-    C *sm1 = ex + (size_t)(CB + c) * region_stride<C>(H, CB);
     for (int i = threadIdx.x; i < a.N2; i += blockDim.x) f2[i] = inv2[i];
     if (threadIdx.x == 0) {
         // PRIN: every thread arrives once a phase, when its copies have landed
@@ -360,80 +300,39 @@ __global__ void __launch_bounds__(MAXT, MINB)
             return cscale(v, sq * f2[r < a.N2 ? r : 0]);
         };
         auto row_needed = [&](int row) { return ((row - rr.x) & (a.n2 - 1)) < rr.y; };
-        if constexpr (DUAL) {
-            // input i = t + e H/E of both halves: y_n and y_n e^{2 pi i n / n2}.
-            // With n2 = 2H the twiddle is e^{2 pi i t / n2} e^{i pi e / E}, negated
-            // for n = i - H: one table read a thread, the rest rotations by
-            // multiples of pi/8 that are constants once the loop over e unrolls.
-            constexpr int TT = (1 << LOGH) / E;
-            const C wt = ldt(&tw[t]);
-            auto ld2 = [&](int i, C &y0, C &y1) {
-                y0 = y1 = cmake((R)0, (R)0);
-                if (!col_ok) return;
-                const int e = (i - t) / TT;
-                const C wi = cmul(wt, cmake((R)c16(e * (8 / E)), (R)s16(e * (8 / E))));
-                if (i < half) {
-                    const C y = coef_nm(i);
-                    y0 = y0 + y;
-                    y1 = y1 + cmul(y, wi);
-                } else if (i >= H - half) {
-                    const C y = coef_nm(i - H);
-                    y0 = y0 + y;
-                    y1 = y1 - cmul(y, wi);
-                }
-                if (HERM && i == half) {
-                    const C y = coef_nm(half);
-                    y0 = y0 + y;
-                    y1 = y1 + cmul(y, ldt(&tw[half]));
-                }
-            };
-            auto st2 = [&](int qq, C z0, C z1) {
-                if (!col_ok) return;
-                if (row_needed(2 * qq)) dst[(size_t)(2 * qq) * a.tpitch] = z0;
-                if (row_needed(2 * qq + 1)) dst[(size_t)(2 * qq + 1) * a.tpitch] = z1;
-            };
-            auto refill = [&]() {
-                if (issuer && a.nbuf == 1 && nxt < a.total) issue(nxt, 0);
-            };
-            line_fft_ct2<LOGH, E>(stw, sm, sm1, t, ld2, st2, refill);
-            __syncthreads();
-        } else {
 #pragma unroll 1
-            for (int s = 0; s < 2; ++s) {
-                auto term = [&](int n) -> C {
-                    C y = coef_nm(n);
-                    if (s) y = cmul(y, ldt(&tw[n & (a.n2 - 1)]));
-                    return y;
-                };
-                auto ld = [&](int i) -> C {
-                    C y = cmake((R)0, (R)0);
-                    if (!col_ok) return y;
-                    if (i < half) y = term(i);
-                    else if (i >= H - half) y = term(i - H);
-                    if (HERM && i == half) y = y + term(half);
-                    return y;
-                };
-                auto st = [&](int qq, C v) {
-                    const int row = 2 * qq + s;
-                    if (col_ok && row_needed(row)) dst[(size_t)row * a.tpitch] = v;
-                };
-                if constexpr (LOGH > 0) line_fft_ct<LOGH, E>(stw, sm, t, ld, st);
-                else line_fft<E>(a.logh, tw, 1, sm, t, ld, st);
-                __syncthreads();
-            }
-            if (a.nbuf == 1 && issuer && nxt < a.total) issue(nxt, 0);
+        for (int s = 0; s < 2; ++s) {
+            auto term = [&](int n) -> C {
+                C y = coef_nm(n);
+                if (s) y = cmul(y, ldt(&tw[n & (a.n2 - 1)]));
+                return y;
+            };
+            auto ld = [&](int i) -> C {
+                C y = cmake((R)0, (R)0);
+                if (!col_ok) return y;
+                if (i < half) y = term(i);
+                else if (i >= H - half) y = term(i - H);
+                if (HERM && i == half) y = y + term(half);
+                return y;
+            };
+            auto st = [&](int qq, C v) {
+                const int row = 2 * qq + s;
+                if (col_ok && row_needed(row)) dst[(size_t)row * a.tpitch] = v;
+            };
+            if constexpr (LOGH > 0) line_fft_ct<LOGH, E>(stw, sm, t, ld, st);
+            else line_fft<E>(a.logh, tw, 1, sm, t, ld, st);
+            __syncthreads();
         }
+        if (a.nbuf == 1 && issuer && nxt < a.total) issue(nxt, 0);
     }
 }
 
 // Per precision: elements per thread E, threads per CTA at most MAXT, resident
 // CTAs MINB the register budget is set for (plain kernel); for the TMA kernel
-// columns per block CB, threads at most TMAXT and TMINB resident CTAs per SM
-// (two CTAs of two columns each keep an SM busy while either waits at a
-// barrier of its transform).
+// columns per block CB, threads at most TMAXT and TMINB resident CTAs per SM.
 template <typename R> struct ThetaCfg;
 template <> struct ThetaCfg<float> {
-    static const int E = DFS_FFT_E, MAXT = 1024, MINB = 1, CB = 2, TMAXT = 512, TMINB = 2;
+    static const int E = DFS_FFT_E, MAXT = 1024, MINB = 1;
 };
 template <> struct ThetaCfg<double> {
     static const int E = DFS_FFT_E, MAXT = 512, MINB = 1, CB = 2, TMAXT = 512, TMINB = 1;
@@ -517,13 +416,11 @@ cudaError_t launch_theta_tma_cb(dfsnufft_plan p, const void *coeffs, int prM, in
     a.in_elems = a.nbox * a.box_rows * CB;
     a.tx_bytes = (unsigned)(sizeof(C) * a.in_elems);
     if (pr && (long long)CB * (prN + 1) > a.in_elems) return cudaErrorNotSupported;
-    // compile-time lengths in FP32 run both halves at once (see k_theta_tma)
-    const bool dual = sizeof(R) == 4 && p->d_stw_theta && a.logh >= 9 && a.logh <= 11;
-    const size_t ex_bytes = sizeof(C) * (size_t)(dual ? 2 : 1) * CB * region_len<C>(H);
+    const size_t ex_bytes = sizeof(C) * (size_t)CB * region_len<C>(H);
     const size_t f2_bytes = sizeof(R) * (size_t)((q.N2 + 3) & ~3) + sizeof(C) * CB;
     const size_t limit = (MINB > 1 ? 226 / MINB : 220) * 1024;
     const size_t in_bytes = sizeof(C) * (size_t)a.in_elems;
-    a.nbuf = !dual && 256 + 2 * in_bytes + ex_bytes + f2_bytes <= limit ? 2 : 1;
+    a.nbuf = 256 + 2 * in_bytes + ex_bytes + f2_bytes <= limit ? 2 : 1;
     const size_t smem = 256 + a.nbuf * in_bytes + ex_bytes + f2_bytes;
     if (smem > limit) return cudaErrorNotSupported;
     CUtensorMap tmap;
@@ -544,13 +441,11 @@ cudaError_t launch_theta_tma_cb(dfsnufft_plan p, const void *coeffs, int prM, in
     return dispatch_theta_tma<R, CB, false>(p, a, tmap, coeffs, smem, grid, threads);
 }
 
-// The configured block width, else (FP64 columns of 8192 fine rows) one column.
+// The configured block width, else (columns of 8192 fine rows) one column.
 template <typename R>
 cudaError_t launch_theta_tma(dfsnufft_plan p, const void *coeffs, int prM, int prN) {
     cudaError_t e = launch_theta_tma_cb<R, ThetaCfg<R>::CB>(p, coeffs, prM, prN);
-    if constexpr (sizeof(R) == 8) {
-        if (e == cudaErrorNotSupported) e = launch_theta_tma_cb<R, 1>(p, coeffs, prM, prN);
-    }
+    if (e == cudaErrorNotSupported) e = launch_theta_tma_cb<R, 1>(p, coeffs, prM, prN);
     return e;
 }
 
@@ -603,8 +498,13 @@ cudaError_t run_theta_plain(dfsnufft_plan p, const ThetaArgs &a, const void *coe
 template <typename R>
 cudaError_t launch_theta(dfsnufft_plan p, const void *coeffs, int prM, int prN) {
     typedef typename CxT<R>::type C;
-    if constexpr (!std::is_same<R, df32>::value) {
+    if constexpr (std::is_same<R, double>::value) {
         cudaError_t e = launch_theta_tma<R>(p, coeffs, prM, prN);
+        if (e != cudaErrorNotSupported) return e;
+        cudaGetLastError();
+    }
+    if constexpr (std::is_same<R, float>::value) {
+        cudaError_t e = dfs_launch_theta_pair(p, coeffs, prM, prN);
         if (e != cudaErrorNotSupported) return e;
         cudaGetLastError();
     }
