@@ -315,9 +315,8 @@ def profile_traffic(kernel, workload):
 
 def set_points_launches(prm):
     """Kernels one set_points launches: one fold for unsorted points; else
-    fold+count, the in-bin row prefix, the two bin-scan passes and the
-    scatter."""
-    return 1 if prm["flags"] & 2 else 5
+    fold+count, the bin scan and the scatter."""
+    return 1 if prm["flags"] & 2 else 3
 
 
 def max_over_ranks(x, ws, device="cpu"):

@@ -57,10 +57,8 @@ __host__ __device__ __forceinline__ C cmul(C a, C b) {
 // Row-block granularity of the "fine rows needed" mask (rows per flag).
 #define DFS_ROW_BLOCK 16
 #define DFS_MAX_ROW_BLOCKS (8192 / DFS_ROW_BLOCK)
-// Bin scan: chunks of DFS_SCAN_CHUNK bins (one CTA each), at most
-// DFS_SCAN_MAXCH chunks (bins <= (8192/8) x DFS_MAX_ROW_BLOCKS).
-#define DFS_SCAN_CHUNK 4096
-#define DFS_SCAN_MAXCH 128
+// Bin scan: chunks of DFS_SCAN_CHUNK bins, one CTA each, a thread a bin.
+#define DFS_SCAN_CHUNK 512
 #define DFS_FFT_MIN_LOG 4
 #define DFS_FFT_MAX_LOG 13
 // Event pairs kept per stage before read_timing must drain them.
@@ -83,7 +81,7 @@ struct dfsnufft_plan_s {
     int *d_emax;                    // per line: largest coefficient exponent (df32.cuh scaling)
     int nbx, nby, nbins;    // interpolation bins
     int bstride;            // per-member stride of the bin arrays: >= nbins + 1, multiple of 4
-    int cstride;            // per-member stride of d_bin_count: bstride + the scan workspace
+    int cstride;            // per-member stride of d_bin_count (dfs_cstride)
     int nch;                // bin-scan chunks, ceil(nbins / DFS_SCAN_CHUNK)
     cudaStream_t stream;
 
@@ -96,9 +94,10 @@ struct dfsnufft_plan_s {
     void *d_stw_phi;        // stage-ordered twiddles of the length-n1/2 phi transforms
     void *d_T;              // theta-pass output, (members x fields) x n2 x dfs_tpitch columns
     void *d_G;              // fine grids (real part), (members x fields) x n2 x n1, plan precision
-    int *d_bin_count;       // members x cstride: counts, then the scan workspace
+    int *d_bin_count;       // members x cstride: scan workspace, then the row counts
     int *d_bin_start;       // members x bstride (nbins + 1 used), member-local positions
-    int *d_task_bin;        // members x bstride: lists of non-empty bins
+    int2 *d_task_bin;       // members x bstride: the non-empty bins in order, (bin, its
+                            // start), then (nbins, the member's points)
     int *d_n_tasks;         // members
     int2 *d_rowrange;           // per member: circular range of needed fine rows (first, count)
     int *d_pofs;                // members + 1 point offsets (device)
@@ -130,9 +129,9 @@ struct dfsnufft_plan_s {
     int64_t n_points, cap_points;   // all members' points
     void *d_urec;           // unsorted folded records (dfs_fold_rec_bytes each): base
                             // cell, rank inside its bin (input order), offsets
-    int2 *d_base;           // sorted: first-tap fine index (i0, j0)
-    void *d_frac;           // sorted: offsets (tx, ty) in plan precision
-    int *d_idx;             // sorted: original point index
+    void *d_base;           // sorted points: FP32 records of 16 bytes (base cell, index,
+                            // offsets), FP64 (base cell, index) pairs (DfsPoints)
+    void *d_frac;           // sorted points, FP64: offsets (tx, ty)
     double *d_pts_stage;    // host-variant staging: 2 x cap_points
     void *d_coef_stage;     // host-variant staging of coefficients
     void *d_val_stage;      // host-variant staging of values
@@ -210,15 +209,69 @@ __host__ __device__ __forceinline__ int dfs_fold_rec_bytes(int dtype) {
     return dtype == DFSNUFFT_F64 ? 24 : 16;
 }
 
-// Ints per member of the count array: counts (bstride), completion counter (4),
-// bin-row flags (DFS_MAX_ROW_BLOCKS bytes), chunk sums and non-empty counts,
-// then from dfs_rowcount_offset the per-row counts of every bin (nbins x
+// Ints per member of the count array: the scan workspace (ticket and completion
+// counters, bin-row flags of DFS_MAX_ROW_BLOCKS bytes, one 64-bit word a scan
+// chunk), then from dfs_rowcount_offset the per-row counts of every bin (nbins x
 // tile_y, bin-major), which order the points inside a bin by fine row.
-__host__ __device__ __forceinline__ int dfs_rowcount_offset(int bstride) {
-    return bstride + 4 + DFS_MAX_ROW_BLOCKS / 4 + 2 * DFS_SCAN_MAXCH;
+__host__ __device__ __forceinline__ int dfs_rowcount_offset(int nbins) {
+    const int chunks = (nbins + DFS_SCAN_CHUNK - 1) / DFS_SCAN_CHUNK;
+    return 4 + DFS_MAX_ROW_BLOCKS / 4 + 2 * ((chunks + 1) & ~1);
 }
-__host__ __device__ __forceinline__ int dfs_cstride(int bstride, int nbins, int tile_y) {
-    return dfs_rowcount_offset(bstride) + ((nbins * tile_y + 3) & ~3);
+__host__ __device__ __forceinline__ int dfs_cstride(int nbins, int tile_y) {
+    return dfs_rowcount_offset(nbins) + ((nbins * tile_y + 3) & ~3);
+}
+
+// The sorted points (or, DFSNUFFT_KEEP_ORDER, the points in the caller's order)
+// as the interpolation reads them: base cell, offsets and the point's index.
+// One 16-byte record in FP32; in FP64 the packed base and index beside the two
+// offsets.  base packs the base cell (bx | by << 16, both below 2^13).
+template <typename R> struct DfsPoints;
+template <> struct DfsPoints<float> {
+    float4 *rec;            // (base, index) as bits, tx, ty
+    __device__ __forceinline__ void load(size_t i, int &base, int &idx, float &tx,
+                                         float &ty) const {
+        const float4 v = __ldg(rec + i);
+        base = __float_as_int(v.x);
+        idx = __float_as_int(v.y);
+        tx = v.z;
+        ty = v.w;
+    }
+    __device__ __forceinline__ void store(size_t i, int base, int idx, float tx, float ty) const {
+        rec[i] = make_float4(__int_as_float(base), __int_as_float(idx), tx, ty);
+    }
+};
+template <> struct DfsPoints<double> {
+    int2 *bi;
+    double2 *off;
+    __device__ __forceinline__ void load(size_t i, int &base, int &idx, double &tx,
+                                         double &ty) const {
+        const int2 b = __ldg(bi + i);
+        const double2 t = __ldg(off + i);
+        base = b.x;
+        idx = b.y;
+        tx = t.x;
+        ty = t.y;
+    }
+    __device__ __forceinline__ void store(size_t i, int base, int idx, double tx,
+                                          double ty) const {
+        bi[i] = make_int2(base, idx);
+        off[i] = make_double2(tx, ty);
+    }
+};
+// Bytes a point of the two buffers.
+__host__ __forceinline__ size_t dfs_point_base_bytes(int dtype) {
+    return dtype == DFSNUFFT_F64 ? sizeof(int2) : sizeof(float4);
+}
+__host__ __forceinline__ size_t dfs_point_frac_bytes(int dtype) {
+    return dtype == DFSNUFFT_F64 ? sizeof(double2) : 0;
+}
+template <typename R> __host__ __forceinline__ DfsPoints<R> dfs_points(const dfsnufft_plan_s *p);
+template <> __host__ __forceinline__ DfsPoints<float> dfs_points<float>(const dfsnufft_plan_s *p) {
+    return DfsPoints<float>{(float4 *)p->d_base};
+}
+template <>
+__host__ __forceinline__ DfsPoints<double> dfs_points<double>(const dfsnufft_plan_s *p) {
+    return DfsPoints<double>{(int2 *)p->d_base, (double2 *)p->d_frac};
 }
 
 // The line window of the next launches: first line and count.

@@ -218,17 +218,16 @@ __device__ void interp_task(const EnsGroup &g, int member, int slot0, unsigned c
     const int p0 = g.pofs[member];
     const int Pk = g.pofs[member + 1] - p0;
     const int ntask = g.n_tasks[member];
-    const int *task_bin = g.task_bin + (size_t)member * g.bstride;
-    const int *bin_start = g.bin_start + (size_t)member * g.bstride;
+    const int2 *tasks = g.task_bin + (size_t)member * g.bstride;
     const float *hc = g.horner;
     for (int slot = slot0; slot < slot0 + ENS_BINS && slot < ntask; ++slot) {
-        const int bin = task_bin[slot];
+        const int bin = tasks[slot].x;
         const int by = bin / g.nbx;
         const int bx = bin - by * g.nbx;
         const int col0 = (bx * g.tile_x - g.c0) & ~1;
         const int row0 = by * g.tile_y - g.c0;
-        const int s = p0 + bin_start[bin];
-        const int e = p0 + bin_start[bin + 1];
+        const int s = p0 + tasks[slot].y;
+        const int e = p0 + tasks[slot + 1].y;
         __syncthreads();                         // the previous bin's reads are done
         const int nq = g.F * TH * Q;
         for (int i = threadIdx.x; i < nq; i += kThreads) {
@@ -244,14 +243,14 @@ __device__ void interp_task(const EnsGroup &g, int member, int slot0, unsigned c
         }
         __syncthreads();
         for (int pi = s + threadIdx.x; pi < e; pi += kThreads) {
-            const int2 b = g.base[pi];
-            const float2 tf = g.frac[pi];
-            const int ox = b.x - col0;
+            int cell, d;
+            float2 tf;
+            g.pts.load(pi, cell, d, tf.x, tf.y);
+            const int ox = (cell & 0xffff) - g.c0 - col0;
             const int odd = ox & 1;
             float w8[WP], wy[W];
             ens_weights<W>(hc, tf.x, tf.y, odd, w8, wy);
-            const int oy = b.y - row0;
-            const int d = g.idx[pi];
+            const int oy = (cell >> 16) - g.c0 - row0;
             for (int ff = 0; ff < g.F; ++ff) {
                 const float2 *tp = reinterpret_cast<const float2 *>(
                     tile + (size_t)ff * tsz + oy * TW + (ox - odd));
@@ -445,7 +444,6 @@ bool dfs_ensemble_group(dfsnufft_plan p, EnsGroup &g) {
     g.T = (float2 *)p->d_T;
     g.G = (float *)p->d_G;
     g.rowrange = p->d_rowrange;
-    g.bin_start = p->d_bin_start;
     g.task_bin = p->d_task_bin;
     g.n_tasks = p->d_n_tasks;
     g.pofs = p->d_pofs;
@@ -455,7 +453,5 @@ bool dfs_ensemble_group(dfsnufft_plan p, EnsGroup &g) {
 // Point records of the group's plan as they stand (set_points may reallocate
 // them when the point count grows).
 void dfs_ensemble_group_points(dfsnufft_plan p, EnsGroup &g) {
-    g.base = p->d_base;
-    g.frac = (const float2 *)p->d_frac;
-    g.idx = p->d_idx;
+    g.pts = dfs_points<float>(p);
 }

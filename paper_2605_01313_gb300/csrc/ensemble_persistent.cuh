@@ -37,10 +37,9 @@ struct EnsGroup {
     float2 *T;                        // theta-pass buffer
     float *G;                         // fine grids
     const int2 *rowrange;
-    const int *bin_start, *task_bin, *n_tasks, *pofs;
-    const int2 *base;                 // sorted point records
-    const float2 *frac;
-    const int *idx;
+    const int2 *task_bin;             // non-empty bins and their starts
+    const int *n_tasks, *pofs;
+    DfsPoints<float> pts;             // sorted points
     const float2 *coef;               // this step's coefficients and values
     float *values;
 };

@@ -32,7 +32,7 @@ namespace {
 
 struct InterpArgs {
     int n1, n2;
-    int tile_x, tile_y, nbx;
+    int tile_x, tile_y, lnbx;   // lnbx = log2 of the bins per bin row
     int c0;
     int F, FG;            // fields per member, fields staged per pass
     int NG;               // field groups per bin, ceil(F / FG)
@@ -40,6 +40,10 @@ struct InterpArgs {
     int bstride;          // per-member stride of the bin arrays
     int fa, fn;           // fields evaluated: fa .. fa + fn - 1 of each member
 };
+
+// Base cell of a point from its record; the first tap sits c0 cells before it.
+__device__ __forceinline__ int cell_x(int cell) { return cell & 0xffff; }
+__device__ __forceinline__ int cell_y(int cell) { return cell >> 16; }
 
 // Kernel weights by Horner's rule: for tap a the weight phi((a - c0) - t) is a
 // degree-W polynomial in s = t - mid (mid = 0 for odd W, 1/2 for even W),
@@ -78,11 +82,8 @@ __device__ __forceinline__ int ends_inward(int i, int n) {
 template <typename R, int W>
 __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_constant__ Horner<R, W> hw,
                                                 const R *__restrict__ grid,
-                                                const int2 *__restrict__ base,
-                                                const R *__restrict__ frac,
-                                                const int *__restrict__ idx,
-                                                const int *__restrict__ bin_start_all,
-                                                const int *__restrict__ task_all,
+                                                DfsPoints<R> pts,
+                                                const int2 *__restrict__ task_all,
                                                 const int *__restrict__ n_tasks,
                                                 const int *__restrict__ pofs,
                                                 R *__restrict__ out_all) {
@@ -98,16 +99,15 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
-    const int *task_bin = task_all + (size_t)k * a.bstride;
-    const int *bin_start = bin_start_all + (size_t)k * a.bstride;
+    const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
-        const int bin = task_bin[task];
-        const int by = bin / a.nbx;
-        const int bx = bin - by * a.nbx;
+        const int2 tk = tasks[task];
+        const int by = tk.x >> a.lnbx;
+        const int bx = tk.x - (by << a.lnbx);
         const int col0 = bx * a.tile_x - a.c0;
         const int row0 = by * a.tile_y - a.c0;
-        const int s = p0 + bin_start[bin];
-        const int e = p0 + bin_start[bin + 1];
+        const int s = p0 + tk.y;
+        const int e = p0 + tasks[task + 1].y;
         for (int f0 = a.fa; f0 < a.fa + a.fn; f0 += a.FG) {
             const int fg = min(a.FG, a.fa + a.fn - f0);
             __syncthreads();
@@ -123,13 +123,13 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
             }
             __syncthreads();
             for (int pi = s + threadIdx.x; pi < e; pi += blockDim.x) {
-                const int2 b = base[pi];
-                R wx[W], wy[W];
-                es_weights<R, W>(frac[2 * pi], hw, wx);
-                es_weights<R, W>(frac[2 * pi + 1], hw, wy);
-                const int ox = b.x - col0;
-                const int oy = b.y - row0;
-                const int dst = idx[pi];
+                int cell, dst;
+                R tx, ty, wx[W], wy[W];
+                pts.load(pi, cell, dst, tx, ty);
+                es_weights<R, W>(tx, hw, wx);
+                es_weights<R, W>(ty, hw, wy);
+                const int ox = cell_x(cell) - a.c0 - col0;
+                const int oy = cell_y(cell) - a.c0 - row0;
                 for (int ff = 0; ff < fg; ++ff) {
                     const R *tp = tile + ff * tsz + oy * TW + ox;
                     R acc = 0;
@@ -203,11 +203,8 @@ template <int W>
 __global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
                                                    const __grid_constant__ HornerDF<W> hw,
                                                    const float2 *__restrict__ grid,
-                                                   const int2 *__restrict__ base,
-                                                   const double *__restrict__ frac,
-                                                   const int *__restrict__ idx,
-                                                   const int *__restrict__ bin_start_all,
-                                                   const int *__restrict__ task_all,
+                                                   DfsPoints<double> pts,
+                                                   const int2 *__restrict__ task_all,
                                                    const int *__restrict__ n_tasks,
                                                    const int *__restrict__ pofs,
                                                    double *__restrict__ out_all,
@@ -222,16 +219,15 @@ __global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
-    const int *task_bin = task_all + (size_t)k * a.bstride;
-    const int *bin_start = bin_start_all + (size_t)k * a.bstride;
+    const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
-        const int bin = task_bin[task];
-        const int by = bin / a.nbx;
-        const int bx = bin - by * a.nbx;
+        const int2 tk = tasks[task];
+        const int by = tk.x >> a.lnbx;
+        const int bx = tk.x - (by << a.lnbx);
         const int col0 = bx * a.tile_x - a.c0;
         const int row0 = by * a.tile_y - a.c0;
-        const int s = p0 + bin_start[bin];
-        const int e = p0 + bin_start[bin + 1];
+        const int s = p0 + tk.y;
+        const int e = p0 + tasks[task + 1].y;
         for (int f0 = a.fa; f0 < a.fa + a.fn; f0 += a.FG) {
             const int fg = min(a.FG, a.fa + a.fn - f0);
             __syncthreads();
@@ -246,14 +242,15 @@ __global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
             }
             __syncthreads();
             for (int pi = s + threadIdx.x; pi < e; pi += blockDim.x) {
-                const int2 b = base[pi];
+                int cell, dst;
+                double tx, ty;
+                pts.load(pi, cell, dst, tx, ty);
                 df32 wx[W];
-                df_weights<W>(frac[2 * pi], hw, wx);
-                const df32 sy = df_offset<W>(frac[2 * pi + 1]);
+                df_weights<W>(tx, hw, wx);
+                const df32 sy = df_offset<W>(ty);
                 const df32 uy = sy * sy;
-                const int ox = b.x - col0;
-                const int oy = b.y - row0;
-                const int dst = idx[pi];
+                const int ox = cell_x(cell) - a.c0 - col0;
+                const int oy = cell_y(cell) - a.c0 - row0;
                 // stencil rows by mirror pairs (bb, W-1-bb), whose y weights come
                 // from one pair of Horner chains; all fields of the group per
                 // row: few live registers
@@ -471,11 +468,8 @@ template <int W>
 __global__ void __launch_bounds__(128) k_interp_f32(InterpArgs a,
                                                     const __grid_constant__ Horner<float, W> hw,
                                                     const float *__restrict__ grid,
-                                                    const int2 *__restrict__ base,
-                                                    const float *__restrict__ frac,
-                                                    const int *__restrict__ idx,
-                                                    const int *__restrict__ bin_start_all,
-                                                    const int *__restrict__ task_all,
+                                                    DfsPoints<float> pts,
+                                                    const int2 *__restrict__ task_all,
                                                     const int *__restrict__ n_tasks,
                                                     const int *__restrict__ pofs,
                                                     float *__restrict__ out_all) {
@@ -492,16 +486,15 @@ __global__ void __launch_bounds__(128) k_interp_f32(InterpArgs a,
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
-    const int *task_bin = task_all + (size_t)k * a.bstride;
-    const int *bin_start = bin_start_all + (size_t)k * a.bstride;
+    const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
-        const int bin = task_bin[task];
-        const int by = bin / a.nbx;
-        const int bx = bin - by * a.nbx;
+        const int2 tk = tasks[task];
+        const int by = tk.x >> a.lnbx;
+        const int bx = tk.x - (by << a.lnbx);
         const int col0 = (bx * a.tile_x - a.c0) & ~1;
         const int row0 = by * a.tile_y - a.c0;
-        const int s = p0 + bin_start[bin];
-        const int e = p0 + bin_start[bin + 1];
+        const int s = p0 + tk.y;
+        const int e = p0 + tasks[task + 1].y;
         for (int f0 = a.fa; f0 < a.fa + a.fn; f0 += a.FG) {
             const int fg = min(a.FG, a.fa + a.fn - f0);
             __syncthreads();
@@ -536,13 +529,14 @@ __global__ void __launch_bounds__(128) k_interp_f32(InterpArgs a,
             }
             __syncthreads();
             for (int pi = s + threadIdx.x; pi < e; pi += blockDim.x) {
-                const int2 b = base[pi];
-                const int ox = b.x - col0;
+                int cell, dst;
+                float tx, ty;
+                pts.load(pi, cell, dst, tx, ty);
+                const int ox = cell_x(cell) - a.c0 - col0;
                 const int odd = ox & 1;
                 float wy[W], w8[WP];
-                paired_weights<W>(frac[2 * pi], frac[2 * pi + 1], odd, hw, w8, wy);
-                const int oy = b.y - row0;
-                const int dst = idx[pi];
+                paired_weights<W>(tx, ty, odd, hw, w8, wy);
+                const int oy = cell_y(cell) - a.c0 - row0;
                 for (int ff = 0; ff < fg; ++ff) {
                     const float2 *tp = reinterpret_cast<const float2 *>(
                         tile + ff * tsz + oy * TW + (ox - odd));
@@ -576,8 +570,14 @@ __global__ void __launch_bounds__(128) k_interp_f32(InterpArgs a,
 // sets both counters back to zero for the next launch.
 //
 // Two stages: while a CTA evaluates its sub-task from stage j & 1, the boxes
-// of the next one it claimed land in the other stage (claimed and issued by
-// thread 0 after the barrier that ends the reads of that stage).  A box starts
+// of the next one it claimed land in the other stage (claimed and issued after
+// the barrier that ends the reads of that stage).  The chain claim -> task entry
+// -> boxes is walked by the first thread of the last warp, which has no points
+// of the remainder when a bin holds a few more than a multiple of the CTA's 128
+// (a bin of a regular grid's departure points holds about 128), and the
+// geometry reaches the other threads through shared memory (68 -> 65 us on 2.1M
+// points and three fields against thread 0 and geometry loaded by every thread;
+// claiming one sub-task further ahead measured 77 us).  A box starts
 // at the bin's first stencil column rounded down to 4 cells (16 bytes, the TMA
 // alignment rule), so a point's first tap sits at column ox in [0, tile_x + 2]
 // of the box and its reads end below tile_x + 2 + WP <= BW.  BWC, when
@@ -592,11 +592,8 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
                                                     const __grid_constant__ Horner<float, W> hw,
                                                     const __grid_constant__ CUtensorMap gmap,
                                                     const float *__restrict__ grid,
-                                                    const int2 *__restrict__ base,
-                                                    const float *__restrict__ frac,
-                                                    const int *__restrict__ idx,
-                                                    const int *__restrict__ bin_start_all,
-                                                    const int *__restrict__ task_all,
+                                                    DfsPoints<float> pts,
+                                                    const int2 *__restrict__ task_all,
                                                     const int *__restrict__ n_tasks,
                                                     const int *__restrict__ pofs,
                                                     float *__restrict__ out_all,
@@ -607,7 +604,10 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char *sb = smem_raw + ((128 - (smem_u32(smem_raw) & 127)) & 127);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sb);
-    int *s_sub = reinterpret_cast<int *>(sb + 16);   // the sub-task staged in each stage
+    // per stage: first column and row of the box, sorted points [z, w) (z < 0:
+    // no more sub-tasks), and the fields staged (first, count)
+    int4 *s_geo = reinterpret_cast<int4 *>(sb + 16);
+    int2 *s_fld = reinterpret_cast<int2 *>(sb + 48);
     float *stage = reinterpret_cast<float *>(sb + 128);
     const int TH = a.tile_y + W - 1;
     const int BWr = BWC ? BWC : a.BW;         // floats per box row
@@ -616,8 +616,7 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int total = n_tasks[k] * a.NG;
-    const int *task_bin = task_all + (size_t)k * a.bstride;
-    const int *bin_start = bin_start_all + (size_t)k * a.bstride;
+    const int2 *tasks = task_all + (size_t)k * a.bstride;
     int *wk = work + 2 * k;
     if (threadIdx.x == 0) {
         mbar_init(&bar[0], 1);
@@ -629,18 +628,28 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
     auto wraps = [&](int col0, int row0) {
         return col0 < 0 || col0 + a.BW > a.n1 || row0 < 0 || row0 + TH > a.n2;
     };
-    auto issue = [&](int sub, int b) {
+    const bool producer = threadIdx.x == blockDim.x - 32;
+    // Claim a sub-task for stage b and start its boxes; false if none is left.
+    auto stage_next = [&](int b) -> bool {
+        int sub = atomicAdd(&wk[0], 1);
+        if (sub >= total) {
+            s_geo[b] = make_int4(0, 0, -1, 0);
+            return false;
+        }
+        sub = ends_inward(sub, total);
         const int task = sub / a.NG;
-        const int f0 = a.fa + (sub - task * a.NG) * a.FG;
-        const int fg = min(a.FG, a.fa + a.fn - f0);
-        const int bin = task_bin[task];
-        const int by = bin / a.nbx;
-        const int bx = bin - by * a.nbx;
+        const int2 tk = tasks[task], tn = tasks[task + 1];
+        const int by = tk.x >> a.lnbx;
+        const int bx = tk.x - (by << a.lnbx);
         const int col0 = (bx * a.tile_x - a.c0) & ~3;
         const int row0 = by * a.tile_y - a.c0;
+        const int f0 = a.fa + (sub - task * a.NG) * a.FG;
+        const int fg = min(a.FG, a.fa + a.fn - f0);
+        s_geo[b] = make_int4(col0, row0, p0 + tk.y, p0 + tn.y);
+        s_fld[b] = make_int2(f0, fg);
         if (wraps(col0, row0)) {
             mbar_arrive_expect_tx(&bar[b], 0);
-            return;
+            return true;
         }
         float *dst = stage + (size_t)b * a.FG * a.box_f;
         fence_proxy_async_smem();
@@ -648,56 +657,33 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
         for (int ff = 0; ff < fg; ++ff)
             tma_load_2d(dst + (size_t)ff * a.box_f, &gmap, col0 >> 1,   // 8-byte units
                         (k * a.F + f0 + ff) * a.n2 + row0, &bar[b]);
+        return true;
     };
     uint32_t ph0 = 0, ph1 = 0;
-    auto claim = [&]() {
-        const int i = atomicAdd(&wk[0], 1);
-        return i >= total ? total : ends_inward(i, total);
-    };
-    if (threadIdx.x == 0) {
-        const int first = claim();
-        s_sub[0] = first;
-        if (first < total) issue(first, 0);
-    }
+    if (producer) stage_next(0);
     __syncthreads();
     for (int it = 0;; ++it) {
         const int cur = it & 1;
-        const int sub = s_sub[cur];
-        if (sub >= total) break;
-        int nxt = total;
-        if (threadIdx.x == 0) {
-            nxt = claim();
-            s_sub[cur ^ 1] = nxt;
-            if (nxt < total) issue(nxt, cur ^ 1);
-        }
-        // geometry and the first point's record, fetched while the boxes land
-        const int task = sub / a.NG;
-        const int f0 = a.fa + (sub - task * a.NG) * a.FG;
-        const int fg = min(a.FG, a.fa + a.fn - f0);
-        const int bin = task_bin[task];
-        const int by = bin / a.nbx;
-        const int bx = bin - by * a.nbx;
-        const int col0 = (bx * a.tile_x - a.c0) & ~3;
-        const int row0 = by * a.tile_y - a.c0;
-        const int s = p0 + bin_start[bin];
-        const int e = p0 + bin_start[bin + 1];
-        int pi = s + threadIdx.x;
-        int2 b = make_int2(0, 0);
+        const int4 geo = s_geo[cur];
+        if (geo.z < 0) break;
+        const int2 fld = s_fld[cur];
+        const bool staged_next = producer && stage_next(cur ^ 1);
+        // the first point's record, fetched while the boxes land
+        const int col0 = geo.x, row0 = geo.y, e = geo.w;
+        const int f0 = fld.x, fg = fld.y;
+        int pi = geo.z + threadIdx.x;
+        int cell = 0, dst = 0;
         float2 t = make_float2(0.f, 0.f);
-        int dst = 0;
-        if (pi < e) {
-            b = base[pi];
-            t = reinterpret_cast<const float2 *>(frac)[pi];
-            dst = idx[pi];
-        }
+        if (pi < e) pts.load(pi, cell, dst, t.x, t.y);
+        float *out = out_all + (size_t)a.F * p0 + (size_t)f0 * Pk;
         const bool ok = mbar_wait_bounded(&bar[cur], cur ? ph1 : ph0);
         if (cur) ph1 ^= 1;
         else ph0 ^= 1;
         if (__syncthreads_or(!ok)) {
-            if (threadIdx.x == 0) {
+            if (producer) {
                 atomicExch(status, DFS_STATUS_TIMEOUT);
                 mbar_wait_bounded(&bar[cur], cur ? ph1 ^ 1 : ph0 ^ 1);
-                if (nxt < total) mbar_wait_bounded(&bar[cur ^ 1], cur ? ph0 : ph1);
+                if (staged_next) mbar_wait_bounded(&bar[cur ^ 1], cur ? ph0 : ph1);
             }
             __syncthreads();
             break;
@@ -720,23 +706,21 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
             __syncthreads();
         }
         while (pi < e) {
-            const int ox = b.x - col0;
-            const int oy = b.y - row0;
-            const int d = dst;
+            const int ox = cell_x(cell) - a.c0 - col0;
+            const int oy = cell_y(cell) - a.c0 - row0;
+            float *o = out + dst;
+            auto next_record = [&]() {         // in flight during this point's sums
+                pi += blockDim.x;
+                if (pi < e) pts.load(pi, cell, dst, t.x, t.y);
+            };
             if constexpr (BWC != 0 && W % 4 == 3) {
                 ExactRow<W> er;
                 float wy[W];
                 exact_weights<W>(t.x, t.y, ox & 3, hw, er, wy);
-                pi += blockDim.x;
-                if (pi < e) {                  // next record in flight during the sums
-                    b = base[pi];
-                    t = reinterpret_cast<const float2 *>(frac)[pi];
-                    dst = idx[pi];
-                }
+                next_record();
                 for (int ff = 0; ff < fg; ++ff) {
                     const float *tp = tile + (size_t)ff * a.box_f + oy * BWr + ox;
-                    out_all[(size_t)a.F * p0 + (size_t)(f0 + ff) * Pk + d] =
-                        exact_sum<W, BWC>(tp, BWr, er, wy);
+                    o[(size_t)ff * Pk] = exact_sum<W, BWC>(tp, BWr, er, wy);
                 }
                 continue;
             }
@@ -744,28 +728,17 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
                 SplitRow<W> sr;
                 float wy[W];
                 split_weights<W>(t.x, t.y, ox & 1, hw, sr, wy);
-                pi += blockDim.x;
-                if (pi < e) {                  // next record in flight during the sums
-                    b = base[pi];
-                    t = reinterpret_cast<const float2 *>(frac)[pi];
-                    dst = idx[pi];
-                }
+                next_record();
                 for (int ff = 0; ff < fg; ++ff) {
                     const float *tp = tile + (size_t)ff * a.box_f + oy * BWr + ox;
-                    out_all[(size_t)a.F * p0 + (size_t)(f0 + ff) * Pk + d] =
-                        split_sum<W>(tp, BWr, sr, wy);
+                    o[(size_t)ff * Pk] = split_sum<W>(tp, BWr, sr, wy);
                 }
                 continue;
             }
             const int odd = ox & 1;
             float w8[WP], wy[W];
             paired_weights<W>(t.x, t.y, odd, hw, w8, wy);
-            pi += blockDim.x;
-            if (pi < e) {                      // next record in flight during the sums
-                b = base[pi];
-                t = reinterpret_cast<const float2 *>(frac)[pi];
-                dst = idx[pi];
-            }
+            next_record();
             for (int ff = 0; ff < fg; ++ff) {
                 const float2 *tp = reinterpret_cast<const float2 *>(
                     tile + (size_t)ff * a.box_f + oy * BWr + (ox - odd));
@@ -780,10 +753,10 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
                     }
                     acc += wy[bb] * rr;
                 }
-                out_all[(size_t)a.F * p0 + (size_t)(f0 + ff) * Pk + d] = acc;
+                o[(size_t)ff * Pk] = acc;
             }
         }
-        __syncthreads();                       // stage cur is free for the claim after next
+        __syncthreads();                       // stage cur is free for the boxes after next
     }
     // the member's last CTA to finish resets its counters for the next launch
     if (threadIdx.x == 0) {
@@ -804,8 +777,7 @@ template <typename R, int W>
 __global__ void __launch_bounds__(256) k_interp_direct(InterpArgs a,
                                                        const __grid_constant__ Horner<R, W> hw,
                                                        const R *__restrict__ grid,
-                                                       const int2 *__restrict__ base,
-                                                       const R *__restrict__ frac,
+                                                       DfsPoints<R> pts,
                                                        const int *__restrict__ pofs,
                                                        R *__restrict__ out_all) {
     constexpr bool PAIR = sizeof(R) == 4 && W <= 8;
@@ -815,8 +787,10 @@ __global__ void __launch_bounds__(256) k_interp_direct(InterpArgs a,
     const int Pk = pofs[k + 1] - p0;
     const int m1 = a.n1 - 1, m2 = a.n2 - 1;
     for (int pl = blockIdx.x * blockDim.x + threadIdx.x; pl < Pk; pl += gridDim.x * blockDim.x) {
-        const int2 b = base[p0 + pl];
-        const R tx = frac[2 * (size_t)(p0 + pl)], ty = frac[2 * (size_t)(p0 + pl) + 1];
+        int cell, own;
+        R tx, ty;
+        pts.load((size_t)p0 + pl, cell, own, tx, ty);
+        const int2 b = make_int2(cell_x(cell) - a.c0, cell_y(cell) - a.c0);
         R *out = out_all + (size_t)a.F * p0 + pl;
         if constexpr (PAIR) {
             const int odd = b.x & 1;
@@ -874,8 +848,7 @@ template <int W>
 __global__ void __launch_bounds__(256) k_interp_wtile(InterpArgs a,
                                                       const __grid_constant__ Horner<float, W> hw,
                                                       const float *__restrict__ grid,
-                                                      const int2 *__restrict__ base,
-                                                      const float *__restrict__ frac,
+                                                      DfsPoints<float> pts,
                                                       const int *__restrict__ pofs,
                                                       float *__restrict__ out_all) {
     constexpr int WP = (W + 2) & ~1;
@@ -894,8 +867,9 @@ __global__ void __launch_bounds__(256) k_interp_wtile(InterpArgs a,
         int2 b = make_int2(0, 0);
         float2 t = make_float2(0.f, 0.f);
         if (live) {
-            b = base[p0 + pl];
-            t = reinterpret_cast<const float2 *>(frac)[p0 + pl];
+            int cell, own;
+            pts.load((size_t)p0 + pl, cell, own, t.x, t.y);
+            b = make_int2(cell_x(cell) - a.c0, cell_y(cell) - a.c0);
         }
         // unwrap around lane 0's cell, then the chunk's box
         const int bx0 = __shfl_sync(0xffffffffu, b.x, 0), by0 = __shfl_sync(0xffffffffu, b.y, 0);
@@ -980,7 +954,8 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
     a.n2 = q.n2;
     a.tile_x = q.tile_x;
     a.tile_y = q.tile_y;
-    a.nbx = p->nbx;
+    a.lnbx = 0;
+    while ((1 << a.lnbx) < p->nbx) ++a.lnbx;
     a.c0 = p->c0;
     a.F = p->n_fields;
     a.bstride = p->bstride;
@@ -1007,12 +982,11 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
             for (int i = 0; i < W; ++i)
                 for (int kk = 0; kk <= W; ++kk) hf.c[i][kk] = (float)hw.c[i][kk];
             k_interp_wtile<W><<<dim3((unsigned)blocks, M), 256, 0, p->stream>>>(
-                a, hf, (const float *)p->d_G, p->d_base, (const float *)p->d_frac, p->d_pofs,
-                (float *)values);
+                a, hf, (const float *)p->d_G, dfs_points<float>(p), p->d_pofs, (float *)values);
             return cudaGetLastError();
         }
         k_interp_direct<R, W><<<dim3((unsigned)blocks, M), 256, 0, p->stream>>>(
-            a, hw, (const R *)p->d_G, p->d_base, (const R *)p->d_frac, p->d_pofs, (R *)values);
+            a, hw, (const R *)p->d_G, dfs_points<R>(p), p->d_pofs, (R *)values);
         return cudaGetLastError();
     }
     if constexpr (sizeof(R) == 4 && W <= 8) {
@@ -1062,11 +1036,9 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
                 if (want < 1) want = 1;
                 return dfs_launch_dependent(
                     kern, dim3((unsigned)want, M), dim3(128), smem, p->stream, a, hf,
-                    p->tmap_G, (const float *)p->d_G, (const int2 *)p->d_base,
-                    (const float *)p->d_frac, (const int *)p->d_idx,
-                    (const int *)p->d_bin_start, (const int *)p->d_task_bin,
-                    (const int *)p->d_n_tasks, (const int *)p->d_pofs, (float *)values,
-                    p->d_status, p->d_work);
+                    p->tmap_G, (const float *)p->d_G, dfs_points<float>(p),
+                    (const int2 *)p->d_task_bin, (const int *)p->d_n_tasks,
+                    (const int *)p->d_pofs, (float *)values, p->d_status, p->d_work);
             }
         }
         // plain loads: tile rows of at most 32 pairs
@@ -1084,8 +1056,8 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
             cudaError_t e = dfs_allow_smem((const void *)k_interp_f32<W>, smem);
             if (e) return e;
             k_interp_f32<W><<<dim3(per, M), 128, smem, p->stream>>>(
-                a, hf, (const float *)p->d_G, p->d_base, (const float *)p->d_frac, p->d_idx,
-                p->d_bin_start, p->d_task_bin, p->d_n_tasks, p->d_pofs, (float *)values);
+                a, hf, (const float *)p->d_G, dfs_points<float>(p), p->d_task_bin, p->d_n_tasks,
+                p->d_pofs, (float *)values);
             return cudaGetLastError();
         }
     }
@@ -1115,8 +1087,7 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
             if (e) return e;
             return dfs_launch_dependent(
                 k_interp_df<W>, dim3(per, M), dim3(256), smem_df, p->stream, a, hd,
-                (const float2 *)p->d_G, (const int2 *)p->d_base, (const double *)p->d_frac,
-                (const int *)p->d_idx, (const int *)p->d_bin_start, (const int *)p->d_task_bin,
+                (const float2 *)p->d_G, dfs_points<double>(p), (const int2 *)p->d_task_bin,
                 (const int *)p->d_n_tasks, (const int *)p->d_pofs, (double *)values,
                 (const int *)p->d_emax);
         }
@@ -1125,10 +1096,9 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
     if (e) return e;
     const int threads = sizeof(R) == 4 ? 128 : 256;
     return dfs_launch_dependent(k_interp<R, W>, dim3(per, M), dim3(threads), smem, p->stream, a,
-                                hw, (const R *)p->d_G, (const int2 *)p->d_base,
-                                (const R *)p->d_frac, (const int *)p->d_idx,
-                                (const int *)p->d_bin_start, (const int *)p->d_task_bin,
-                                (const int *)p->d_n_tasks, (const int *)p->d_pofs, (R *)values);
+                                hw, (const R *)p->d_G, dfs_points<R>(p),
+                                (const int2 *)p->d_task_bin, (const int *)p->d_n_tasks,
+                                (const int *)p->d_pofs, (R *)values);
 }
 
 template <typename R, int W>
