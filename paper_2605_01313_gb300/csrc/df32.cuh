@@ -1,12 +1,9 @@
 // Double-single arithmetic for the FP64 plans: a value carried as an unevaluated
 // sum hi + lo of two FP32 numbers (|lo| <= ulp(hi) / 2, 48 significant bits),
 // so that FP64-accurate work runs on the FP32 units, which GB300 has at 64 times
-// its FP64 rate.  Error-free transformations (Knuth's TwoSum, the FMA-based
-// TwoProduct) and the compensated dot product of Ogita, Rump and Oishi (Dot2):
-// a sum of products accumulated this way carries an error of about
-// (n u)^2 sum |x_i y_i| (u = 2^-24) before its final rounding.  The operations
-// use the _rn intrinsics so that no product is contracted into a neighbouring
-// addition, which would break the transformations.
+// its FP64 rate.  Built on error-free transformations (Knuth's TwoSum, the
+// FMA-based TwoProduct); the operations use the _rn intrinsics so that no product
+// is contracted into a neighbouring addition, which would break them.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -38,17 +35,6 @@ __device__ __forceinline__ df32 two_sum(float a, float b) {
 __device__ __forceinline__ df32 quick_two_sum(float a, float b) {
     const float s = __fadd_rn(a, b);
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-
-// a * s + c in double-single (one Horner step).
-__device__ __forceinline__ df32 df_mul_add(df32 a, df32 s, df32 c) {
-    const float p = __fmul_rn(a.hi, s.hi);
-    float e = fmaf(a.hi, s.hi, -p);
-    e = fmaf(a.hi, s.lo, e);
-    e = fmaf(a.lo, s.hi, e);
-    df32 t = two_sum(p, c.hi);
-    t.lo = __fadd_rn(t.lo, __fadd_rn(e, c.lo));
-    return quick_two_sum(t.hi, t.lo);
 }
 
 // Arithmetic on double-single values ("sloppy" addition: the low parts are
@@ -88,16 +74,6 @@ __device__ __forceinline__ dfc ldt(const dfc *p) {
 }
 __device__ __forceinline__ float2 ldt(const float2 *p) { return __ldg(p); }
 __device__ __forceinline__ double2 ldt(const double2 *p) { return __ldg(p); }
-
-// One term of a compensated dot product: (r, c) += x * y with x, y double-single;
-// r is the running FP32 sum, c collects the rounding errors and the low parts.
-__device__ __forceinline__ void dot2_step(float &r, float &c, df32 x, df32 y) {
-    const float p = __fmul_rn(x.hi, y.hi);
-    const float e = fmaf(x.hi, y.hi, -p);
-    const df32 t = two_sum(r, p);
-    r = t.hi;
-    c = fmaf(x.hi, y.lo, fmaf(x.lo, y.hi, __fadd_rn(c, __fadd_rn(t.lo, e))));
-}
 
 // A double as hi + lo: hi holds the top 24 bits of the significand (truncated),
 // lo the remaining 29 rounded to 24, by integer operations on the bit pattern

@@ -147,19 +147,61 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
     }
 }
 
-// ---- FP64 plans in double-single arithmetic (df32.cuh)
+// ---- FP64 plans
 //
-// The fine grid holds (hi, lo) FP32 pairs (written so by the phi pass), the
-// Horner coefficients are split the same way, the weights are evaluated by
-// double-single Horner steps and every stencil sum is a compensated dot
-// product (Dot2): about 10 FP32 operations a tap instead of one FP64 FMA, on
-// units that run 64 times faster, with an error of about (w u)^2 sum |w g|
-// (u = 2^-24, a few 1e-13 of the value for smooth fields).
-#define DFS_DF_FG 4            // fields a CTA of k_interp_df stages at once, at most
+// The fine grid holds (hi, lo) FP32 pairs (written so by the phi pass), and the
+// kernel weights are double-single (df32.cuh).  The stencil sums are taken in
+// fixed point: GB300 multiplies 32 x 32 bits into a 64-bit sum in two cycles a
+// warp instruction on each scheduler (mad.wide.s32, measured), so a tap takes
+// three such products, 6 cycles, where a compensated floating-point step
+// (Dot2) takes 12 instructions.  The sums are exact in integers and the
+// operands keep more bits than double-single has:
+//
+//   tile values  g = S (gh 2^-30 + gl 2^-59),  |gh| < 2^30, |gl| <= 2^28, S the
+//                power of two above the largest |g| of the staged tile (halo
+//                included) of that field: an error of 2^-60 S;
+//   weights      w = wh 2^-22 + wl 2^-51,  |wh| <= 2^22, |wl| <= 1.25 2^28.
+//
+// A row's sum of wh gh (below 2^55) and the sum of its cross products wl gh +
+// wh gl (below 2^63 for w <= 16; wl gl stays below 2^-79 S) join as an integer of
+// units 2^-57 S, which the y weights sum the same way; the point's value is
+// assembled into an FP64 bit pattern by integer operations (GB300's FP64 units
+// run at 1/64 rate, and the conversions alone took 7% of the kernel).  Against
+// the tile's largest value the quantisation adds about 2e-16.  A tile that holds
+// a non-finite value gives NaN.
+#define DFS_FX_FG 4            // fields a CTA of k_interp_fx stages at once, at most
 
 template <int W> struct HornerDF {
     float hi[W][W + 1], lo[W][W + 1];
 };
+
+// One chain of a weight polynomial in u = s^2, coefficients k0, k0 - 2, .. k1 of
+// tap a, by compensated Horner's rule (Graillat, Langlois and Louvet): an FP32
+// recurrence whose product and sum errors, with the low parts of the
+// coefficients and of u, run through a second one.  The first TOP steps are
+// plain FP32: on |s| <= 1/2 what they add is smaller than the weight by 1e-8 and
+// more, and their rounding stays below 4e-16 of the largest weight (TOP from the
+// fitted coefficients of both oversampling factors: 2 for w >= 15, 1 for w >= 13).
+template <int W>
+__device__ __forceinline__ df32 df_chain(const HornerDF<W> &h, int a, int k0, int k1, df32 u) {
+    constexpr int TOP = W >= 15 ? 2 : W >= 13 ? 1 : 0;
+    float e = h.hi[a][k0];
+    float err = TOP ? 0.f : h.lo[a][k0];
+#pragma unroll
+    for (int k = k0 - 2; k >= k1; k -= 2) {
+        if (k0 - k <= 2 * TOP) {
+            e = fmaf(e, u.hi, h.hi[a][k]);
+            continue;
+        }
+        const float p = __fmul_rn(e, u.hi);
+        float c = fmaf(e, u.hi, -p);
+        const df32 t = two_sum(p, h.hi[a][k]);
+        c = __fadd_rn(__fadd_rn(c, t.lo), h.lo[a][k]);
+        err = fmaf(err, u.hi, fmaf(e, u.lo, c));
+        e = t.hi;
+    }
+    return quick_two_sum(e, err);
+}
 
 // The kernel is even, so tap W-1-a at s is tap a at -s: with tap a's
 // polynomial split into even and odd parts in u = s^2, P_a(+-s) = E(u) +- s O(u)
@@ -167,14 +209,8 @@ template <int W> struct HornerDF {
 template <int W>
 __device__ __forceinline__ void df_pair(const HornerDF<W> &h, int a, df32 s, df32 u, df32 &lo,
                                         df32 &hi) {
-    constexpr int KE = W - (W & 1);           // highest even power
-    constexpr int KO = W - 1 + (W & 1);       // highest odd power
-    df32 e = {h.hi[a][KE], h.lo[a][KE]};
-#pragma unroll
-    for (int k = KE - 2; k >= 0; k -= 2) e = df_mul_add(e, u, df32{h.hi[a][k], h.lo[a][k]});
-    df32 o = {h.hi[a][KO], h.lo[a][KO]};
-#pragma unroll
-    for (int k = KO - 2; k >= 1; k -= 2) o = df_mul_add(o, u, df32{h.hi[a][k], h.lo[a][k]});
+    const df32 e = df_chain<W>(h, a, W - (W & 1), 0, u);
+    const df32 o = df_chain<W>(h, a, W - 1 + (W & 1), 1, u);
     const df32 so = s * o;
     lo = e + so;                               // tap a
     hi = e - so;                               // tap W-1-a
@@ -185,36 +221,77 @@ __device__ __forceinline__ df32 df_offset(double t) {
     return split_double(t - (W % 2 == 0 ? 0.5 : 0.0));
 }
 
-template <int W>
-__device__ __forceinline__ void df_weights(double t, const HornerDF<W> &h, df32 *wv) {
-    const df32 s = df_offset<W>(t);
-    const df32 u = s * s;
-#pragma unroll
-    for (int a = 0; a < (W + 1) / 2; ++a) {
-        df32 lo, hi;
-        df_pair<W>(h, a, s, u, lo, hi);
-        wv[a] = lo;
-        if (W - 1 - a != a) wv[W - 1 - a] = hi;
-    }
+// A weight's two integers: wh by adding 3 (whose binade has a spacing of 2^-22),
+// the exact remainder and the low part together as wl.
+__device__ __forceinline__ void fix_weight(df32 w, int &h, int &l) {
+    const float m = __fadd_rn(w.hi, 3.f);
+    h = __float_as_int(m) - 0x40400000;
+    const float r = __fsub_rn(w.hi, __fsub_rn(m, 3.f));
+    l = __float2int_rn(__fmul_rn(__fadd_rn(r, w.lo), 0x1p51f));
 }
 
-// As k_interp, with the tile of (hi, lo) pairs.
+// A tile value times k = 2^30 / S as (gh, gl): the integer part of hi k, then
+// the integer part and the fraction of what is left with lo k (at most 65).
+__device__ __forceinline__ int2 fix_cell(float2 g, float k) {
+    const float x = __fmul_rn(g.x, k);
+    const int h = __float2int_rn(x);
+    const float y = fmaf(g.y, k, __fsub_rn(x, __int2float_rn(h)));
+    const float m = __fadd_rn(y, 12582912.f);            // 1.5 2^23: y to an integer
+    const float f = __fsub_rn(y, __fsub_rn(m, 12582912.f));
+    return make_int2(h + (__float_as_int(m) - 0x4b400000), __float2int_rn(__fmul_rn(f, 0x1p29f)));
+}
+
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    return (long long)a * b + c;
+}
+
+// v 2^ex as an FP64 number (rounded half up) by integer operations; results
+// outside the normal range by scalbn.
+__device__ __forceinline__ double fix_value(long long v, int ex) {
+    if (v == 0) return 0.0;
+    unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)a);
+    const int e = 1023 + 63 - lz + ex;
+    if (e < 1 || e > 2045) return scalbn((double)v, ex);
+    a <<= lz;
+    const unsigned long long bits =
+        ((unsigned long long)(e - 1) << 52) + (a >> 11) + ((a >> 10) & 1);
+    return __longlong_as_double((long long)(bits | ((unsigned long long)v & (1ull << 63))));
+}
+
+// One CTA a bin: the tile and its halo of up to DFS_FX_FG fields arrive by
+// 16-byte asynchronous copies (rows start on an even column), each thread finds
+// the largest magnitude of the cells it copied and, once the CTA knows the
+// tile's, converts those cells in place.  Then a thread a point: the x weights
+// once, the y weights by mirror pairs of stencil rows, all fields per row.  A row
+// of W cells is read as aligned pairs and one or two single cells at its ends by
+// the parity of its first column, so no cell outside the stencil is read and a
+// quarter-warp's 16-byte reads of neighbouring points do not conflict.
+// Two CTAs an SM (98 KB of tiles for three fields at w = 14, 128-cell bins).
 template <int W>
-__global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
-                                                   const __grid_constant__ HornerDF<W> hw,
-                                                   const float2 *__restrict__ grid,
-                                                   DfsPoints<double> pts,
-                                                   const int2 *__restrict__ task_all,
-                                                   const int *__restrict__ n_tasks,
-                                                   const int *__restrict__ pofs,
-                                                   double *__restrict__ out_all,
-                                                   const int *__restrict__ emax) {
+__global__ void __launch_bounds__(256, 2) k_interp_fx(InterpArgs a,
+                                                      const __grid_constant__ HornerDF<W> hw,
+                                                      const float2 *__restrict__ grid,
+                                                      DfsPoints<double> pts,
+                                                      const int2 *__restrict__ task_all,
+                                                      const int *__restrict__ n_tasks,
+                                                      const int *__restrict__ pofs,
+                                                      double *__restrict__ out_all,
+                                                      const int *__restrict__ emax) {
     dfs_grid_wait();
+    constexpr int NS = W % 2 == 0 ? 2 : 1;     // single cells a row
+    constexpr int NP = (W - NS) / 2;           // pairs a row
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float2 *tile = reinterpret_cast<float2 *>(smem_raw);
+    int2 *tile = reinterpret_cast<int2 *>(smem_raw);
+    __shared__ unsigned s_max[DFS_FX_FG];
     const int TH = a.tile_y + W - 1;
-    const int TW = a.tile_x + W - 1;
+    const int TW = (a.tile_x + W + 1) & ~1;
+    const int Q = TW / 2;                      // 16-byte chunks a row
+    const int nq = TH * Q;
     const int tsz = TH * TW;
+    // this thread's first chunk of a tile, and the step to its next one
+    const int r_first = threadIdx.x / Q, c_first = threadIdx.x - r_first * Q;
+    const int r_step = blockDim.x / Q, c_step = blockDim.x - r_step * Q;
     const int k = blockIdx.y;
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
@@ -224,51 +301,131 @@ __global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
         const int2 tk = tasks[task];
         const int by = tk.x >> a.lnbx;
         const int bx = tk.x - (by << a.lnbx);
-        const int col0 = bx * a.tile_x - a.c0;
+        const int col0 = (bx * a.tile_x - a.c0) & ~1;
         const int row0 = by * a.tile_y - a.c0;
         const int s = p0 + tk.y;
         const int e = p0 + tasks[task + 1].y;
         for (int f0 = a.fa; f0 < a.fa + a.fn; f0 += a.FG) {
             const int fg = min(a.FG, a.fa + a.fn - f0);
+            __syncthreads();                   // the tiles of the pass before are consumed
+            if (threadIdx.x < DFS_FX_FG) s_max[threadIdx.x] = 0;
+            for (int ff = 0; ff < fg; ++ff) {
+                const float2 *g = grid + (size_t)(k * a.F + f0 + ff) * a.n2 * a.n1;
+                int r = r_first, c = c_first;
+                for (int i = threadIdx.x; i < nq; i += blockDim.x) {
+                    const int gr = (row0 + r) & (a.n2 - 1);
+                    const int gc = (col0 + 2 * c) & (a.n1 - 1);
+                    cp_async_16(tile + ff * tsz + 2 * i, g + (size_t)gr * a.n1 + gc);
+                    r += r_step;
+                    c += c_step;
+                    if (c >= Q) {
+                        c -= Q;
+                        ++r;
+                    }
+                }
+            }
+            cp_async_wait_all();
+            __syncthreads();                   // s_max is zero
+            for (int ff = 0; ff < fg; ++ff) {
+                const float4 *t4 = reinterpret_cast<const float4 *>(tile + ff * tsz);
+                unsigned m = 0;                // as bits: NaN above infinity above all else
+                for (int i = threadIdx.x; i < nq; i += blockDim.x) {
+                    const float4 v = t4[i];
+                    m = max(m, max(__float_as_uint(v.x) & 0x7fffffffu,
+                                   __float_as_uint(v.z) & 0x7fffffffu));
+                }
+                m = __reduce_max_sync(0xffffffffu, m);
+                if ((threadIdx.x & 31) == 0) atomicMax(&s_max[ff], m);
+            }
             __syncthreads();
-            for (int rr = threadIdx.x >> 5; rr < fg * TH; rr += blockDim.x >> 5) {
-                const int ff = rr / TH;
-                const int r = rr - ff * TH;
-                const int gr = (row0 + r) & (a.n2 - 1);
-                const float2 *src = grid + ((size_t)(k * a.F + f0 + ff) * a.n2 + gr) * a.n1;
-                float2 *dst = tile + ff * tsz + r * TW;
-                for (int cc = threadIdx.x & 31; cc < TW; cc += 32)
-                    dst[cc] = src[(col0 + cc) & (a.n1 - 1)];
+            for (int ff = 0; ff < fg; ++ff) {
+                // S = 2^(ue - 126), the power of two above the largest magnitude (at
+                // least 2^-90: below it the field is zero next to the line's largest
+                // coefficient, which is in [1, 2))
+                const int ue = max((int)(s_max[ff] >> 23), 36);
+                if (ue >= 255) continue;
+                const float kf = __int_as_float((127 + 30 + 126 - ue) << 23);
+                int4 *t4 = reinterpret_cast<int4 *>(tile + ff * tsz);
+                for (int i = threadIdx.x; i < nq; i += blockDim.x) {
+                    const float4 v = *reinterpret_cast<const float4 *>(t4 + i);
+                    const int2 x = fix_cell(make_float2(v.x, v.y), kf);
+                    const int2 y = fix_cell(make_float2(v.z, v.w), kf);
+                    t4[i] = make_int4(x.x, x.y, y.x, y.y);
+                }
             }
             __syncthreads();
             for (int pi = s + threadIdx.x; pi < e; pi += blockDim.x) {
                 int cell, dst;
                 double tx, ty;
                 pts.load(pi, cell, dst, tx, ty);
-                df32 wx[W];
-                df_weights<W>(tx, hw, wx);
-                const df32 sy = df_offset<W>(ty);
-                const df32 uy = sy * sy;
                 const int ox = cell_x(cell) - a.c0 - col0;
                 const int oy = cell_y(cell) - a.c0 - row0;
-                // stencil rows by mirror pairs (bb, W-1-bb), whose y weights come
-                // from one pair of Horner chains; all fields of the group per
-                // row: few live registers
-                float r2[DFS_DF_FG], c2[DFS_DF_FG];
+                const int odd = ox & 1;
+                // x weights in read order: pairs from tap `odd` on, then the singles
+                // (tap 0 or the last but one of an even W; the last tap)
+                int wph[2 * NP + 1], wpl[2 * NP + 1], wsh[NS], wsl[NS];
+                {
+                    const df32 sx = df_offset<W>(tx);
+                    const df32 ux = sx * sx;
+                    int wh[W], wl[W];
 #pragma unroll
-                for (int ff = 0; ff < DFS_DF_FG; ++ff) r2[ff] = c2[ff] = 0.f;
-                auto row = [&](int bb, df32 wyb) {
+                    for (int t = 0; t < (W + 1) / 2; ++t) {
+                        df32 lo, hi;
+                        df_pair<W>(hw, t, sx, ux, lo, hi);
+                        fix_weight(lo, wh[t], wl[t]);
+                        if (W - 1 - t != t) fix_weight(hi, wh[W - 1 - t], wl[W - 1 - t]);
+                    }
 #pragma unroll
-                    for (int ff = 0; ff < DFS_DF_FG; ++ff) {
+                    for (int i = 0; i < 2 * NP; ++i) {
+                        wph[i] = odd ? wh[i + 1] : wh[i];
+                        wpl[i] = odd ? wl[i + 1] : wl[i];
+                    }
+                    wsh[0] = odd ? wh[0] : wh[W - NS];
+                    wsl[0] = odd ? wl[0] : wl[W - NS];
+                    if (NS == 2) {
+                        wsh[NS - 1] = wh[W - 1];
+                        wsl[NS - 1] = wl[W - 1];
+                    }
+                }
+                const df32 sy = df_offset<W>(ty);
+                const df32 uy = sy * sy;
+                const int2 *tp0 = tile + oy * TW + ox;
+                const int o1 = odd ? 0 : W - NS;
+                long long yh[DFS_FX_FG], yl[DFS_FX_FG];
+#pragma unroll
+                for (int ff = 0; ff < DFS_FX_FG; ++ff) yh[ff] = yl[ff] = 0;
+                auto row = [&](int bb, df32 wy) {
+                    int vh, vl;
+                    fix_weight(wy, vh, vl);
+#pragma unroll
+                    for (int ff = 0; ff < DFS_FX_FG; ++ff) {
                         if (ff >= fg) break;
-                        const float2 *tp = tile + ff * tsz + (oy + bb) * TW + ox;
-                        float r = 0.f, c = 0.f;
+                        const int2 *tp = tp0 + ff * tsz + bb * TW;
+                        const int4 *tq = reinterpret_cast<const int4 *>(tp + odd);
+                        long long h = 0, c0 = 0, c1 = 0;
+                        auto tap = [&](int xh, int xl, int gh, int gl) {
+                            h = mad_wide(xh, gh, h);
+                            c0 = mad_wide(xl, gh, c0);
+                            c1 = mad_wide(xh, gl, c1);
+                        };
 #pragma unroll
-                        for (int aa = 0; aa < W; ++aa) {
-                            const float2 g = tp[aa];
-                            dot2_step(r, c, wx[aa], df32{g.x, g.y});
+                        for (int i = 0; i < NP; ++i) {
+                            const int4 g = tq[i];
+                            tap(wph[2 * i], wpl[2 * i], g.x, g.y);
+                            tap(wph[2 * i + 1], wpl[2 * i + 1], g.z, g.w);
                         }
-                        dot2_step(r2[ff], c2[ff], wyb, quick_two_sum(r, c));
+                        const int2 g0 = tp[o1];
+                        tap(wsh[0], wsl[0], g0.x, g0.y);
+                        if (NS == 2) {
+                            const int2 g1 = tp[W - 1];
+                            tap(wsh[NS - 1], wsl[NS - 1], g1.x, g1.y);
+                        }
+                        // the row in units of 2^-57 S, as rh 2^29 + rl
+                        const long long r = (h << 5) + ((c0 + c1) >> 24);
+                        const int rh = (int)(r >> 29), rl = (int)r & 0x1fffffff;
+                        yh[ff] = mad_wide(vh, rh, yh[ff]);
+                        yl[ff] = mad_wide(vl, rh, yl[ff]);
+                        yl[ff] = mad_wide(vh, rl, yl[ff]);
                     }
                 };
 #pragma unroll 1
@@ -278,13 +435,20 @@ __global__ void __launch_bounds__(256) k_interp_df(InterpArgs a,
                     row(bb, wlo);
                     if (W - 1 - bb != bb) row(W - 1 - bb, whi);
                 }
-                // back to the caller's scale: the line was carried as c 2^-s
+                const bool bad = !(tx == tx);          // an unfoldable point: NaN offsets
+                double *out = out_all + (size_t)a.F * p0 + (size_t)f0 * Pk + dst;
 #pragma unroll
-                for (int ff = 0; ff < DFS_DF_FG; ++ff)
-                    if (ff < fg)
-                        out_all[(size_t)a.F * p0 + (size_t)(f0 + ff) * Pk + dst] =
-                            ((double)r2[ff] + (double)c2[ff]) *
-                            df_pow2(df_line_shift(emax[k * a.F + f0 + ff]));
+                for (int ff = 0; ff < DFS_FX_FG; ++ff)
+                    if (ff < fg) {
+                        const int ue = max((int)(s_max[ff] >> 23), 36);
+                        // units of 2^-58 S, back to the caller's scale: the line was
+                        // carried as c 2^-s
+                        const long long v = (yh[ff] << 8) + (yl[ff] >> 21);
+                        const int ex = ue - 126 - 58 + df_line_shift(emax[k * a.F + f0 + ff]);
+                        out[(size_t)ff * Pk] = bad || ue >= 255
+                                                   ? __longlong_as_double(0x7ff8000000000000LL)
+                                                   : fix_value(v, ex);
+                    }
             }
         }
     }
@@ -1081,12 +1245,20 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
                     hd.hi[i][kk] = (float)c;
                     hd.lo[i][kk] = (float)(c - (double)hd.hi[i][kk]);
                 }
-            if (a.FG > DFS_DF_FG) a.FG = DFS_DF_FG;
-            const size_t smem_df = per_field * a.FG;
-            cudaError_t e = dfs_allow_smem((const void *)k_interp_df<W>, smem_df);
+            const size_t tile =
+                sizeof(int2) * (size_t)(q.tile_y + W - 1) * ((q.tile_x + W + 1) & ~1);
+            // fields a CTA holds at once: as many as leave two CTAs an SM (one if
+            // none does), the passes over the fields evened out
+            a.FG = (int)(112 * 1024 / tile);
+            if (a.FG < 1) a.FG = 1;
+            if (a.FG > DFS_FX_FG) a.FG = DFS_FX_FG;
+            const int passes = (a.fn + a.FG - 1) / a.FG;
+            a.FG = (a.fn + passes - 1) / passes;
+            const size_t smem_fx = tile * a.FG;
+            cudaError_t e = dfs_allow_smem((const void *)k_interp_fx<W>, smem_fx);
             if (e) return e;
             return dfs_launch_dependent(
-                k_interp_df<W>, dim3(per, M), dim3(256), smem_df, p->stream, a, hd,
+                k_interp_fx<W>, dim3(per, M), dim3(256), smem_fx, p->stream, a, hd,
                 (const float2 *)p->d_G, dfs_points<double>(p), (const int2 *)p->d_task_bin,
                 (const int *)p->d_n_tasks, (const int *)p->d_pofs, (double *)values,
                 (const int *)p->d_emax);
