@@ -2,13 +2,11 @@
 // through the packed FP32 instructions of sm_100 and later (add / mul / fma on
 // a 64-bit register pair, .f32x2).
 //
-// GB300 runs a packed instruction at half the rate of a scalar one (measured:
-// 2.0 against 1.0 cycles a warp instruction on each of an SM's four
-// schedulers), so packing buys no arithmetic rate; it halves the issue slots
-// the arithmetic takes, which is what bounded the two passes (58% of the issue
-// slots busy with FP32 arithmetic, index arithmetic, shared-memory exchanges and
-// table loads competing for them).  The exchanges move one 16-byte element (both
-// transforms' complex values) where two 8-byte ones moved before.  Against the
+// Packing halves the issue slots the arithmetic takes (f32x2.cuh), which is what
+// bounded the two passes (58% of the issue slots busy, FP32 and index
+// arithmetic, shared-memory exchanges and table loads competing for them).  The
+// exchanges move one 16-byte element (both transforms' complex values) where two
+// 8-byte ones moved before.  Against the
 // scalar two-line form (2048 x 1024 grid, three fields): theta pass 65 -> 57 us,
 // phi pass 58 -> 40 us.
 //
@@ -17,42 +15,10 @@
 // multiplication by +-i swaps the operands of a subtraction.
 #pragma once
 
+#include "f32x2.cuh"
 #include "fft_core.cuh"
 
 namespace dfs_fft {
-
-typedef unsigned long long f32x2;          // (low word, high word) = (value 0, value 1)
-
-__device__ __forceinline__ f32x2 pk(float a, float b) {
-    f32x2 r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ float2 unpk(f32x2 v) {
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ f32x2 padd(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 psub(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 pmul(f32x2 a, f32x2 b) {
-    f32x2 r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ f32x2 pfma(f32x2 a, f32x2 b, f32x2 c) {
-    f32x2 r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
 
 struct __align__(16) PairC {
     f32x2 x, y;

@@ -150,25 +150,33 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
 // ---- FP64 plans
 //
 // The fine grid holds (hi, lo) FP32 pairs (written so by the phi pass), and the
-// kernel weights are double-single (df32.cuh).  The stencil sums are taken in
-// fixed point: GB300 multiplies 32 x 32 bits into a 64-bit sum in two cycles a
-// warp instruction on each scheduler (mad.wide.s32, measured), so a tap takes
-// three such products, 6 cycles, where a compensated floating-point step
-// (Dot2) takes 12 instructions.  The sums are exact in integers and the
-// operands keep more bits than double-single has:
+// kernel weights are double-single (df32.cuh).  The stencil sums are taken with
+// the leading product in fixed point: one 32 x 32 product into a 64-bit sum
+// (IMAD.WIDE, about 4 cycles a warp instruction on one of the two FMA pipes,
+// measured) adds exactly, and the two cross products, 2^-30 of it, are added in
+// FP32.  A tap is then a wide product, a byte permutation and two FMAs, spread
+// over the FMA pipes and the ALU, where a compensated floating-point step (Dot2)
+// takes 12 instructions and a product of two-limb integers three wide products.
+// 2.1M points, three fields, w = 14: 1122 us with Dot2, 836 with two-limb
+// integers, 726 in this form (65% of the issue slots; more warps an SM, narrower
+// bins and the fields' sums interleaved were no faster).  Of its 8600
+// instructions per 32 points the weights take a third and the tiles' staging a
+// twelfth.
 //
-//   tile values  g = S (gh 2^-30 + gl 2^-59),  |gh| < 2^30, |gl| <= 2^28, S the
-//                power of two above the largest |g| of the staged tile (halo
-//                included) of that field: an error of 2^-60 S;
-//   weights      w = wh 2^-22 + wl 2^-51,  |wh| <= 2^22, |wl| <= 1.25 2^28.
+//   tile values  g = S (gh 2^-30 + gl),  |gh| < 2^30, |gl| <= 2^-31, S the power
+//                of two above the largest |g| of the staged tile (halo included)
+//                of that field; stored as (gl, gh + 2^30);
+//   weights      w = wh 2^-30 + wl,  |wl| <= 2^-31.
 //
-// A row's sum of wh gh (below 2^55) and the sum of its cross products wl gh +
-// wh gl (below 2^63 for w <= 16; wl gl stays below 2^-79 S) join as an integer of
-// units 2^-57 S, which the y weights sum the same way; the point's value is
-// assembled into an FP64 bit pattern by integer operations (GB300's FP64 units
-// run at 1/64 rate, and the conversions alone took 7% of the kernel).  Against
-// the tile's largest value the quantisation adds about 2e-16.  A tile that holds
-// a non-finite value gives NaN.
+// With sum w <= 3.3 (w <= 16) a row's sum of wh (gh + 2^30) stays below 2^63; it
+// starts from -2^30 sum wh, which takes the bias out.  The cross products are
+// wl g, whose g comes from the top 23 bits of gh + 2^30 set under the exponent
+// of 2^23 (a byte permutation; its bias 1.5 2^23 is taken out by the sum's start),
+// and w gl; their rounding stays near 2^-50 S.  A row joins as an integer of units
+// 2^-60 S, the rows are summed with the y weights the same way, and the point's
+// value is assembled into an FP64 bit pattern by integer operations (GB300's FP64
+// units run at 1/64 rate, and the conversions alone took 7% of the kernel).  A
+// tile that holds a non-finite value gives NaN.
 #define DFS_FX_FG 4            // fields a CTA of k_interp_fx stages at once, at most
 
 template <int W> struct HornerDF {
@@ -221,24 +229,22 @@ __device__ __forceinline__ df32 df_offset(double t) {
     return split_double(t - (W % 2 == 0 ? 0.5 : 0.0));
 }
 
-// A weight's two integers: wh by adding 3 (whose binade has a spacing of 2^-22),
-// the exact remainder and the low part together as wl.
-__device__ __forceinline__ void fix_weight(df32 w, int &h, int &l) {
-    const float m = __fadd_rn(w.hi, 3.f);
-    h = __float_as_int(m) - 0x40400000;
-    const float r = __fsub_rn(w.hi, __fsub_rn(m, 3.f));
-    l = __float2int_rn(__fmul_rn(__fadd_rn(r, w.lo), 0x1p51f));
+// v = (hi, lo) times k as an integer, and the fraction f left, |f| <= 1/2: the
+// integer part of hi k, then that of what is left with lo k (at most 65).
+__device__ __forceinline__ int fix_split(df32 v, float k, float &f) {
+    const float x = __fmul_rn(v.hi, k);
+    const int h = __float2int_rn(x);
+    const float y = fmaf(v.lo, k, __fsub_rn(x, __int2float_rn(h)));
+    const float m = __fadd_rn(y, 12582912.f);            // 1.5 2^23: y to an integer
+    f = __fsub_rn(y, __fsub_rn(m, 12582912.f));
+    return h + (__float_as_int(m) - 0x4b400000);
 }
 
-// A tile value times k = 2^30 / S as (gh, gl): the integer part of hi k, then
-// the integer part and the fraction of what is left with lo k (at most 65).
+// A tile value as (gl, gh + 2^30), k = 2^30 / S.
 __device__ __forceinline__ int2 fix_cell(float2 g, float k) {
-    const float x = __fmul_rn(g.x, k);
-    const int h = __float2int_rn(x);
-    const float y = fmaf(g.y, k, __fsub_rn(x, __int2float_rn(h)));
-    const float m = __fadd_rn(y, 12582912.f);            // 1.5 2^23: y to an integer
-    const float f = __fsub_rn(y, __fsub_rn(m, 12582912.f));
-    return make_int2(h + (__float_as_int(m) - 0x4b400000), __float2int_rn(__fmul_rn(f, 0x1p29f)));
+    float f;
+    const int h = fix_split(df32{g.x, g.y}, k, f);
+    return make_int2(__float_as_int(__fmul_rn(f, 0x1p-30f)), h + (1 << 30));
 }
 
 __device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
@@ -362,70 +368,94 @@ __global__ void __launch_bounds__(256, 2) k_interp_fx(InterpArgs a,
                 const int oy = cell_y(cell) - a.c0 - row0;
                 const int odd = ox & 1;
                 // x weights in read order: pairs from tap `odd` on, then the singles
-                // (tap 0 or the last but one of an even W; the last tap)
-                int wph[2 * NP + 1], wpl[2 * NP + 1], wsh[NS], wsl[NS];
+                // (tap 0 or the last but one of an even W; the last tap); wh, and
+                // (w, wl 2^-22)
+                int ph[2 * NP + 1], sh[NS];
+                float2 pw[2 * NP + 1], sw[NS];
+                long long h0 = 0;              // the starts of a row's sums
+                float c0 = 0.f;
                 {
                     const df32 sx = df_offset<W>(tx);
                     const df32 ux = sx * sx;
-                    int wh[W], wl[W];
+                    int wh[W];
+                    float wf[W], wl[W];
+                    auto put = [&](int t, df32 w) {
+                        float f;
+                        wh[t] = fix_split(w, 0x1p30f, f);
+                        wf[t] = w.hi;
+                        wl[t] = __fmul_rn(f, 0x1p-52f);
+                        h0 -= wh[t];
+                        c0 = fmaf(-12582912.f, wl[t], c0);
+                    };
 #pragma unroll
                     for (int t = 0; t < (W + 1) / 2; ++t) {
                         df32 lo, hi;
                         df_pair<W>(hw, t, sx, ux, lo, hi);
-                        fix_weight(lo, wh[t], wl[t]);
-                        if (W - 1 - t != t) fix_weight(hi, wh[W - 1 - t], wl[W - 1 - t]);
+                        put(t, lo);
+                        if (W - 1 - t != t) put(W - 1 - t, hi);
                     }
+                    h0 <<= 30;
+                    auto pick = [&](int t1, int t0, int &h, float2 &p) {
+                        h = odd ? wh[t1] : wh[t0];
+                        p = make_float2(odd ? wf[t1] : wf[t0], odd ? wl[t1] : wl[t0]);
+                    };
 #pragma unroll
-                    for (int i = 0; i < 2 * NP; ++i) {
-                        wph[i] = odd ? wh[i + 1] : wh[i];
-                        wpl[i] = odd ? wl[i + 1] : wl[i];
-                    }
-                    wsh[0] = odd ? wh[0] : wh[W - NS];
-                    wsl[0] = odd ? wl[0] : wl[W - NS];
-                    if (NS == 2) {
-                        wsh[NS - 1] = wh[W - 1];
-                        wsl[NS - 1] = wl[W - 1];
-                    }
+                    for (int i = 0; i < 2 * NP; ++i) pick(i + 1, i, ph[i], pw[i]);
+                    pick(0, W - NS, sh[0], sw[0]);
+                    if (NS == 2) pick(W - 1, W - 1, sh[NS - 1], sw[NS - 1]);
                 }
                 const df32 sy = df_offset<W>(ty);
                 const df32 uy = sy * sy;
                 const int2 *tp0 = tile + oy * TW + ox;
                 const int o1 = odd ? 0 : W - NS;
-                long long yh[DFS_FX_FG], yl[DFS_FX_FG];
+                // the values: yh 2^-58 S + yc S
+                long long yh[DFS_FX_FG];
+                float yc[DFS_FX_FG];
 #pragma unroll
-                for (int ff = 0; ff < DFS_FX_FG; ++ff) yh[ff] = yl[ff] = 0;
+                for (int ff = 0; ff < DFS_FX_FG; ++ff) {
+                    yh[ff] = 0;
+                    yc[ff] = 0.f;
+                }
                 auto row = [&](int bb, df32 wy) {
-                    int vh, vl;
-                    fix_weight(wy, vh, vl);
+                    float f;
+                    const int vh = fix_split(wy, 0x1p30f, f);
+                    const float vl = __fmul_rn(f, 0x1p-58f);       // times r 2^-32
+                    const float vf = __fmul_rn(wy.hi, 0x1p-60f);   // times r mod 2^32
 #pragma unroll
                     for (int ff = 0; ff < DFS_FX_FG; ++ff) {
                         if (ff >= fg) break;
                         const int2 *tp = tp0 + ff * tsz + bb * TW;
                         const int4 *tq = reinterpret_cast<const int4 *>(tp + odd);
-                        long long h = 0, c0 = 0, c1 = 0;
-                        auto tap = [&](int xh, int xl, int gh, int gl) {
+                        long long h = h0;
+                        float cx = 0.f, cy = c0;
+                        auto tap = [&](int xh, float2 xw, int gl, int gh) {
                             h = mad_wide(xh, gh, h);
-                            c0 = mad_wide(xl, gh, c0);
-                            c1 = mad_wide(xh, gl, c1);
+                            const int t = (int)__byte_perm(gh, 0x4b, 0x4321);
+                            cx = fmaf(xw.x, __int_as_float(gl), cx);
+                            cy = fmaf(xw.y, __int_as_float(t), cy);
                         };
 #pragma unroll
                         for (int i = 0; i < NP; ++i) {
                             const int4 g = tq[i];
-                            tap(wph[2 * i], wpl[2 * i], g.x, g.y);
-                            tap(wph[2 * i + 1], wpl[2 * i + 1], g.z, g.w);
+                            tap(ph[2 * i], pw[2 * i], g.x, g.y);
+                            tap(ph[2 * i + 1], pw[2 * i + 1], g.z, g.w);
                         }
                         const int2 g0 = tp[o1];
-                        tap(wsh[0], wsl[0], g0.x, g0.y);
+                        tap(sh[0], sw[0], g0.x, g0.y);
                         if (NS == 2) {
                             const int2 g1 = tp[W - 1];
-                            tap(wsh[NS - 1], wsl[NS - 1], g1.x, g1.y);
+                            tap(sh[NS - 1], sw[NS - 1], g1.x, g1.y);
                         }
-                        // the row in units of 2^-57 S, as rh 2^29 + rl
-                        const long long r = (h << 5) + ((c0 + c1) >> 24);
-                        const int rh = (int)(r >> 29), rl = (int)r & 0x1fffffff;
+                        // the row as r = rh 2^32 + rl in units of 2^-60 S (the cross
+                        // products, below 2^-27 S, to 2^-57 S)
+                        const float2 cc = make_float2(cx, cy);
+                        const int ci = __float2int_rn(__fmul_rn(__fadd_rn(cc.x, cc.y), 0x1p57f));
+                        const long long r = mad_wide(ci, 8, h);
+                        const int rh = (int)(r >> 32);
+                        const unsigned rl = (unsigned)r;
                         yh[ff] = mad_wide(vh, rh, yh[ff]);
-                        yl[ff] = mad_wide(vl, rh, yl[ff]);
-                        yl[ff] = mad_wide(vh, rl, yl[ff]);
+                        yc[ff] = fmaf(vf, __uint2float_rn(rl),
+                                      fmaf(vl, __int2float_rn(rh), yc[ff]));
                     }
                 };
 #pragma unroll 1
@@ -442,8 +472,10 @@ __global__ void __launch_bounds__(256, 2) k_interp_fx(InterpArgs a,
                     if (ff < fg) {
                         const int ue = max((int)(s_max[ff] >> 23), 36);
                         // units of 2^-58 S, back to the caller's scale: the line was
-                        // carried as c 2^-s
-                        const long long v = (yh[ff] << 8) + (yl[ff] >> 21);
+                        // carried as c 2^-s; a tile of zeros gives zero (the biases
+                        // cancel to rounding only)
+                        const long long v =
+                            s_max[ff] ? yh[ff] + __float2ll_rn(__fmul_rn(yc[ff], 0x1p58f)) : 0;
                         const int ex = ue - 126 - 58 + df_line_shift(emax[k * a.F + f0 + ff]);
                         out[(size_t)ff * Pk] = bad || ue >= 255
                                                    ? __longlong_as_double(0x7ff8000000000000LL)
