@@ -116,6 +116,8 @@ struct dfsnufft_plan_s {
     int *d_parity;              // fields: +1 scalar / -1 wind component (grid input)
     int h_parity[64];           // the parities last uploaded
     int parity_set;
+    double horner[16 * 17];     // kernel weight polynomials (dfsnufft_es_horner), kept so
+                                // that a launch does not fit them again
     int num_sms;                // multiprocessors of the plan's device
     CUtensorMap tmap_G;         // 2-D map of d_G (8-byte elements), box set by the interpolation
     int tmap_G_ok;              // tmap_G is valid (FP32 plans that own their buffers)

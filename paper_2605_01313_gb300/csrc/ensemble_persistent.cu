@@ -432,9 +432,7 @@ bool dfs_ensemble_group(dfsnufft_plan p, EnsGroup &g) {
     g.bstride = p->bstride;
     g.c0 = p->c0;
     g.W = q.w;
-    double hc[8 * 9];
-    dfsnufft_es_horner(q.w, q.beta, hc);
-    for (int i = 0; i < q.w * (q.w + 1); ++i) g.horner[i] = (float)hc[i];
+    for (int i = 0; i < q.w * (q.w + 1); ++i) g.horner[i] = (float)p->horner[i];
     g.inv1 = (const float *)p->d_inv1;
     g.inv2 = (const float *)p->d_inv2;
     g.tw1 = (const float2 *)p->d_tw1;

@@ -101,6 +101,7 @@ extern "C" int dfsnufft_execute_noalloc(int n_lon, int n_lat, double tol, int dt
     p.bstride = (p.nbins + 4) & ~3;
     p.cstride = dfs_cstride(p.nbins, prm.tile_y);
     p.nch = (p.nbins + DFS_SCAN_CHUNK - 1) / DFS_SCAN_CHUNK;
+    dfsnufft_es_horner(prm.w, prm.beta, p.horner);
     p.n_members = 1;
     p.n_points = n_points;
     p.cap_points = n_points;

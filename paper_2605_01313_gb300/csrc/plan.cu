@@ -558,6 +558,7 @@ static int plan_create_impl(int n_members, int n_lon, int n_lat, double tol, int
     p->stream = (cudaStream_t)stream;
     p->herm = (prm.flags & DFSNUFFT_REAL_FIELDS) ? 1 : 0;
     p->keep_order = (prm.flags & DFSNUFFT_KEEP_ORDER) ? 1 : 0;
+    dfsnufft_es_horner(prm.w, prm.beta, p->horner);
     // FP64 with sorted points: fine grid as double-single pairs, interpolation
     // on the FP32 units in double-single arithmetic
     p->gdf = (dtype == DFSNUFFT_F64 && !p->keep_order) ? 1 : 0;
