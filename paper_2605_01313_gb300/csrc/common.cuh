@@ -79,6 +79,9 @@ struct dfsnufft_plan_s {
     void *d_df_stw_theta;           // and (length n2) for the theta pass
     void *d_df_stw_half;            // and (length n2/2) for the forward column pass
     int *d_emax;                    // per line: largest coefficient exponent (df32.cuh scaling)
+    int *d_cexp;                    // and per column of T (lines x dfs_tpitch), when the theta
+                                    // pass scales each column by its own
+    int colscale;                   // the last theta pass did so
     int nbx, nby, nbins;    // interpolation bins
     int bstride;            // per-member stride of the bin arrays: >= nbins + 1, multiple of 4
     int cstride;            // per-member stride of d_bin_count (dfs_cstride)
@@ -294,6 +297,8 @@ cudaError_t dfs_launch_phi_pass(dfsnufft_plan p);
 // without launching, for the shapes they do not take.
 cudaError_t dfs_launch_theta_pair(dfsnufft_plan p, const void *coeffs, int prM, int prN);
 cudaError_t dfs_launch_phi_pair(dfsnufft_plan p);
+// The double-single form (fft_theta_df.cu), likewise.
+cudaError_t dfs_launch_theta_df(dfsnufft_plan p, const void *coeffs);
 // Largest FP64 exponent of each of lines line0 .. line0 + lines - 1 into
 // p->d_emax (the double-single scaling of df32.cuh): every one of the
 // line_elems complex values of a line, or (herm) those a real-field theta pass

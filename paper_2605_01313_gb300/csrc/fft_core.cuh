@@ -5,6 +5,8 @@
 // at compile time, fully unrolled; used for the large transforms).
 #pragma once
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "df32.cuh"
 #include "tma.cuh"
@@ -38,8 +40,35 @@ __device__ __forceinline__ C tw16(C a) {
     } else {
         typedef decltype(a.x) R;
         constexpr R c = (R)c16(k), s = (R)s16(k);
-        return cmake(a.x * c - a.y * s, a.x * s + a.y * c);
+        if constexpr (std::is_same<C, dfc>::value) {
+            constexpr df32 h(c16(2));
+            // odd multiples of pi/4: sums before products
+            if constexpr (k == 2) {
+                return dfc{add_lazy(a.x, -a.y) * h, add_lazy(a.x, a.y) * h};
+            } else if constexpr (k == 6) {
+                return dfc{add_lazy(-a.x, -a.y) * h, add_lazy(a.x, -a.y) * h};
+            } else if constexpr (k == 10) {
+                return dfc{add_lazy(a.y, -a.x) * h, add_lazy(-a.x, -a.y) * h};
+            } else if constexpr (k == 14) {
+                return dfc{add_lazy(a.x, a.y) * h, add_lazy(a.y, -a.x) * h};
+            } else {
+                return cmul(a, dfc{c, s});
+            }
+        } else {
+            return cmake(a.x * c - a.y * s, a.x * s + a.y * c);
+        }
     }
+}
+
+// Sum and difference of a butterfly whose half size is H; only the last level
+// (H = 1) of a double-single step normalises them.
+template <int H, typename C> __device__ __forceinline__ C bf_add(C a, C b) {
+    if constexpr (std::is_same<C, dfc>::value && H > 1) return add_lazy(a, b);
+    else return a + b;
+}
+template <int H, typename C> __device__ __forceinline__ C bf_sub(C a, C b) {
+    if constexpr (std::is_same<C, dfc>::value && H > 1) return sub_lazy(a, b);
+    else return a - b;
 }
 
 // In-place DFT of size R (power of two <= 16), sign +1, on the registers
@@ -53,8 +82,8 @@ __device__ __forceinline__ void dif_step(C *v) {
             constexpr int i = K + (B * 2 * H + P) * S;
             constexpr int j = i + H * S;
             const C a = v[i], c = v[j];
-            v[i] = a + c;
-            v[j] = tw16<P * (8 / H)>(a - c);
+            v[i] = bf_add<H>(a, c);
+            v[j] = tw16<P * (8 / H)>(bf_sub<H>(a, c));
             dif_step<R, K, S, H, B, P + 1>(v);
         } else {
             dif_step<R, K, S, H, B + 1, 0>(v);
@@ -227,9 +256,11 @@ __device__ __forceinline__ void ct_butterfly(C *v, int t, const C *__restrict__ 
     }
 }
 
-template <int LOGN, int E, int LNS, typename C, class St>
+// The stages from log2(Ns) = LNS on.  after_first_barrier() runs on every thread
+// after the barrier that ends the first stage.
+template <int LOGN, int E, int LNS, typename C, class St, class Hook>
 __device__ __forceinline__ void ct_stages(C *v, int t, const C *__restrict__ stw, C *sm,
-                                          St &st) {
+                                          St &st, Hook &after_first_barrier) {
     constexpr int LE = E == 16 ? 4 : E == 8 ? 3 : 2;
     constexpr int REM = LOGN - LNS;
     if constexpr (REM > 0) {
@@ -237,13 +268,14 @@ __device__ __forceinline__ void ct_stages(C *v, int t, const C *__restrict__ stw
         constexpr int T = (1 << LOGN) / E;
         if constexpr (LNS > 0) {
             __syncthreads();
+            if constexpr (LNS == LE) after_first_barrier();
 #pragma unroll
             for (int e = 0; e < E; ++e) v[e] = sm[spad<C>(t + e * T)];
             __syncthreads();
         }
         ct_butterfly<(1 << LR), E, 0, (1 << LNS), stage_table_offset(LOGN, E, LNS), T,
                      REM == LR>(v, t, stw, sm, st);
-        ct_stages<LOGN, E, LNS + LR>(v, t, stw, sm, st);
+        ct_stages<LOGN, E, LNS + LR>(v, t, stw, sm, st, after_first_barrier);
     }
 }
 
@@ -256,7 +288,8 @@ __device__ __forceinline__ void line_fft_ct(const C *__restrict__ stw, C *sm, in
     C v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = ld(t + e * T);
-    ct_stages<LOGN, E, 0>(v, t, stw, sm, st);
+    auto none = [] {};
+    ct_stages<LOGN, E, 0>(v, t, stw, sm, st, none);
 }
 
 // ---- two lines at once (compile-time length)

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
     k_phi_pass(PhiArgs a, const typename CxT<R>::type *__restrict__ in,
                const typename CxT<R>::type *__restrict__ tw,
                const typename CxT<R>::type *__restrict__ stw, const int2 *__restrict__ rowrange,
-               R *__restrict__ grid) {
+               R *__restrict__ grid, const int *__restrict__ cexp, int *__restrict__ emax) {
     dfs_grid_wait();
     typedef typename CxT<R>::type C;
     const int row0 = blockIdx.x * a.CB;
@@ -60,7 +60,38 @@ __global__ void __launch_bounds__(MAXT, MINB)
     const int nmask = a.n1 - 1;
     C *sm = smem + (size_t)c * region_len<C>(M);
     C *srow = smem + (size_t)a.CB * region_len<C>(M) + (size_t)c * a.tcols;
-    for (int i = t; i < a.tcols; i += T) srow[i] = t_load(src, row, i, a.tpitch);
+    bool scaled = false;
+    if constexpr (std::is_same<R, df32>::value) {
+        // T's columns each carry their own power of two (cexp): the line's is the
+        // largest, and each column is brought to it as it is staged
+        scaled = cexp != nullptr;
+        if (scaled) {
+            __shared__ int s_emax;
+            const int *ce = cexp + (size_t)f * a.tpitch;
+            if (threadIdx.x == 0) s_emax = 0;
+            int m = 0;
+            for (int i = threadIdx.x; i < a.tcols; i += blockDim.x) m = max(m, ce[i]);
+            m = __reduce_max_sync(__activemask(), m);
+            __syncthreads();
+            if ((threadIdx.x & 31) == 0) atomicMax(&s_emax, m);
+            __syncthreads();
+            const int em = s_emax;
+            if (threadIdx.x == 0) emax[f] = em;             // every CTA writes the same
+            const int sl = df_line_shift(em);
+            for (int i = t; i < a.tcols; i += T) {
+                const int d = df_line_shift(ce[i]) - sl;    // at most 0 for finite lines
+                const float k = em >= 0x7ff ? 1.f
+                                : ce[i] == 0 || d < -126 ? 0.f
+                                                         : __int_as_float((127 + d) << 23);
+                C v = t_load(src, row, i, a.tpitch);
+                v.x = df32(v.x.hi * k, v.x.lo * k);
+                v.y = df32(v.y.hi * k, v.y.lo * k);
+                srow[i] = v;
+            }
+        }
+    }
+    if (!scaled)
+        for (int i = t; i < a.tcols; i += T) srow[i] = t_load(src, row, i, a.tpitch);
     __syncthreads();
     auto hval = [&](int k) -> C {              // real-field rows: H_k, k taken mod n1
         k &= nmask;
@@ -135,7 +166,9 @@ cudaError_t run_phi_df(dfsnufft_plan p, const PhiArgs &a, size_t smem, dim3 grid
                                 dim3(threads), smem, p->stream, a, (const C *)p->d_T,
                                 (const C *)(dfr ? p->d_df_tw1 : p->d_tw1),
                                 (const C *)(dfr ? p->d_df_stw_phi : p->d_stw_phi),
-                                (const int2 *)p->d_rowrange, (R *)p->d_G);
+                                (const int2 *)p->d_rowrange, (R *)p->d_G,
+                                (const int *)(dfr && p->colscale ? p->d_cexp : nullptr),
+                                p->d_emax);
 }
 
 // FP64 plans whose interpolation runs in double-single (p->gdf) take the DF form.

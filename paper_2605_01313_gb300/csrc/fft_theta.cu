@@ -26,8 +26,8 @@
 // e^{2 pi i n s / n2} e^{2 pi i n q / (n2/2)}, s = 0, 1 (the modes fit in n2/2;
 // when n2 = 2 N2 the two Nyquist modes n = -N2/2 and n = +N2/2 of a real-field
 // plan share index N2/2 and are added there).  k_theta_pass is the plain-load
-// version: FP64 plans in double-single arithmetic, and the shapes the other two
-// do not take (unaligned coefficient pointer, CTA or shared-memory limits).
+// version: FP64 plans' partial-regularity input, and the shapes the others
+// (FP64 plans in double-single arithmetic: fft_theta_df.cu) do not take (unaligned coefficient pointer, CTA or shared-memory limits).
 #include <type_traits>
 
 #include "coef_map.cuh"
@@ -337,10 +337,7 @@ template <> struct ThetaCfg<float> {
 template <> struct ThetaCfg<double> {
     static const int E = DFS_FFT_E, MAXT = 512, MINB = 1, CB = 2, TMAXT = 512, TMINB = 1;
 };
-// Double-single: two CTAs of one column each per SM (64 registers a thread, a
-// few bytes spilled; 70 KB of shared memory each), which hides the latency of
-// the strided coefficient loads better than one CTA at 101 registers (C3 FP64
-// theta pass 413 -> 342 us).
+// Double-single: two CTAs of one column each per SM.
 template <> struct ThetaCfg<df32> {
     static const int E = DFS_FFT_E, MAXT = 512, MINB = 2, CB = 1, TMAXT = 512, TMINB = 1;
 };
@@ -468,22 +465,7 @@ cudaError_t run_theta_plain(dfsnufft_plan p, const ThetaArgs &a, const void *coe
     typedef typename CxT<R>::type C;
     constexpr int MAXT = ThetaCfg<R>::MAXT, MINB = ThetaCfg<R>::MINB;
     if constexpr (std::is_same<R, df32>::value) {
-        // FP64 coefficients, double-single factors and twiddles; lengths 2^10 ..
-        // 2^12 at compile time with the double-single stage-ordered table
-        if constexpr (E == DFS_FFT_E) {
-            switch (p->d_df_stw_theta ? a.logn2 : 0) {
-                case 10:
-                    return run_theta_df<R, E, MAXT, MINB, HERM, PRIN, 10>(p, a, coeffs, smem,
-                                                                          grid, threads);
-                case 11:
-                    return run_theta_df<R, E, MAXT, MINB, HERM, PRIN, 11>(p, a, coeffs, smem,
-                                                                          grid, threads);
-                case 12:
-                    return run_theta_df<R, E, MAXT, MINB, HERM, PRIN, 12>(p, a, coeffs, smem,
-                                                                          grid, threads);
-                default: break;
-            }
-        }
+        // FP64 coefficients, double-single factors and twiddles
         return run_theta_df<R, E, MAXT, MINB, HERM, PRIN, 0>(p, a, coeffs, smem, grid, threads);
     } else {
         cudaError_t e = allow_smem(k_theta_pass<R, E, MAXT, MINB, HERM, PRIN>, smem);
@@ -579,6 +561,11 @@ static cudaError_t launch_coef_maxexp(dfsnufft_plan p, const void *coeffs, int p
 
 cudaError_t dfs_launch_theta_pass(dfsnufft_plan p, const void *coeffs, int prM, int prN) {
     if (p->gdf) {                                  // FP64 in double-single
+        p->colscale = 0;
+        if (prM < 0) {
+            const cudaError_t e = dfs_launch_theta_df(p, coeffs);
+            if (e != cudaErrorNotSupported) return e;
+        }
         cudaError_t e = launch_coef_maxexp(p, coeffs, prM, prN);
         if (e) return e;
         return launch_theta<df32>(p, coeffs, prM, prN);

@@ -323,7 +323,7 @@ static void release(dfsnufft_plan p) {
                      (void **)&p->d_pts_stage, &p->d_coef_stage, &p->d_val_stage,
                      &p->d_df_tw1, &p->d_df_tw2, &p->d_df_inv1, &p->d_df_inv2,
                      &p->d_df_stw_phi, &p->d_df_stw_theta, &p->d_df_stw_half,
-                     (void **)&p->d_emax};
+                     (void **)&p->d_emax, (void **)&p->d_cexp};
     for (size_t i = 0; i < sizeof(bufs) / sizeof(bufs[0]); ++i) dfs_free(bufs[i]);
     free(p->h_pofs);
     p->h_pofs = nullptr;
@@ -610,6 +610,9 @@ static int plan_create_impl(int n_members, int n_lon, int n_lat, double tol, int
     if (rc == DFSNUFFT_OK && p->gdf) rc = upload_df_tables(p);
     if (rc == DFSNUFFT_OK && p->gdf)
         rc = dfs_alloc(p, (void **)&p->d_emax, sizeof(int) * nf, "line exponents");
+    if (rc == DFSNUFFT_OK && p->gdf)
+        rc = dfs_alloc(p, (void **)&p->d_cexp, sizeof(int) * nf * dfs_tpitch(p->herm, prm.N1),
+                       "column exponents");
     if (rc == DFSNUFFT_OK && (prm.flags & DFSNUFFT_GAUSS_GRID)) {
         // samples on Gauss-Legendre latitudes: the solve matrices, in the theta-pass
         // buffer's room for the class matrices
