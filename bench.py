@@ -313,10 +313,12 @@ def profile_traffic(kernel, workload):
     return None
 
 
-def set_points_launches(prm):
-    """Kernels one set_points launches: one fold for unsorted points; else
-    fold+count, the bin scan and the scatter."""
-    return 1 if prm["flags"] & 2 else 3
+def set_points_launches(prm, n_points):
+    """Kernels one set_points of n_points a member launches: one for unsorted
+    points and for small members (points.cu, k_points_small); else fold+count, the
+    bin scan and the scatter."""
+    keys = prm["n1"] // prm["tile_x"] * prm["n2"]
+    return 1 if prm["flags"] & 2 or (n_points <= 4096 and keys <= 8192) else 3
 
 
 def max_over_ranks(x, ws, device="cpu"):
@@ -636,12 +638,15 @@ def measure(args, name, wl, ws, rank, dev, serving, cpu_seconds=None):
         # grid input: the two forward passes (Gauss-Legendre: longitude pass,
         # latitude solve, coefficient mapping; the FP32 solve is our tcgen05
         # kernel, the FP64 one cuBLAS DGEMM, not counted); FP64 plans in
-        # double-single: the exponent reductions of the coefficients (and samples)
-        "gpu_launches": (set_points_launches(prm) + 3
+        # double-single: the exponent reductions of the samples, and of the
+        # coefficients where the theta pass does not find them itself (partial-
+        # regularity input, 8192 fine rows)
+        "gpu_launches": (set_points_launches(prm, P) + 3
                          + ((3 if gauss is not None and wl.dtype == "f32" else 2)
                             if grid_in else 0)
                          + (2 if sl is not None else 0)
-                         + ((1 + (1 if grid_in and gauss is None else 0))
+                         + ((int(pr_in or prm["n2"] > 4096)
+                             + (1 if grid_in and gauss is None else 0))
                             if wl.dtype == "f64" and not prm["flags"] & 2 else 0))
                         * args.steps,
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
@@ -866,7 +871,8 @@ def measure_ensemble(args, name, ws, rank, dev, cpu_seconds):
                   "value": weak_scaling_value(ws, total_pf, args.steps, p_total), "unit": UNIT,
                   "options": pers_note,
                   "gpu_launches_per_step": sum(
-                      set_points_launches(nufft.dfsnufft_plan_get_params(pens.plan_handle(gi)))
+                      set_points_launches(nufft.dfsnufft_plan_get_params(pens.plan_handle(gi)),
+                                          max(pts[gi][2]))
                       for gi in range(len(groups))) + 1,
                   "error": {"rel_linf_first_member_32_points": p_err, "bound": 2e-5,
                             "ok": max(p_err.values()) <= 2e-5}}
@@ -897,7 +903,7 @@ def measure_ensemble(args, name, ws, rank, dev, cpu_seconds):
     sp_launches = []
     for gi, (m, n_lon, n_lat) in enumerate(groups):
         prm = nufft.dfsnufft_plan_get_params(ens.plan_handle(gi))
-        sp_launches.append(set_points_launches(prm))
+        sp_launches.append(set_points_launches(prm, max(pts[gi][2])))
         st = nufft.dfsnufft_plan_point_stats(ens.plan_handle(gi))
         step_bytes += sum(stage_bytes(prm, 3 * m, sum(pts[gi][2]), st["rows_needed"]).values())
     pk, pk_kind = peaks()

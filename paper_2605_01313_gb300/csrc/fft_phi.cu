@@ -220,6 +220,8 @@ cudaError_t launch_phi(dfsnufft_plan p) {
     if (cb > DFS_ROW_BLOCK) cb = DFS_ROW_BLOCK;
     const size_t per_row = sizeof(C) * (size_t)(region_len<C>(M) + a.tcols);
     while (cb > 1 && per_row * cb > 160 * 1024) cb >>= 1;
+    // few rows: fewer a CTA (down to a warp), so that they spread over the SMs
+    while (cb > 1 && cb * T > 32 && (q.n2 / cb) * lines < p->num_sms) cb >>= 1;
     a.CB = cb;
     const size_t smem = per_row * cb;
     const dim3 grid(q.n2 / cb, lines);

@@ -39,6 +39,7 @@ struct InterpArgs {
     int BW, box_f;        // TMA box width (cells, multiple of 4), floats per staged box
     int bstride;          // per-member stride of the bin arrays
     int fa, fn;           // fields evaluated: fa .. fa + fn - 1 of each member
+    int parts;            // CTAs a bin (k_interp_fx)
 };
 
 // Base cell of a point from its record; the first tap sits c0 cells before it.
@@ -303,14 +304,21 @@ __global__ void __launch_bounds__(256, 2) k_interp_fx(InterpArgs a,
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
     const int2 *tasks = task_all + (size_t)k * a.bstride;
-    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+    for (int sub = blockIdx.x; sub < ntask * a.parts; sub += gridDim.x) {
+        const int task = sub / a.parts;
         const int2 tk = tasks[task];
         const int by = tk.x >> a.lnbx;
         const int bx = tk.x - (by << a.lnbx);
         const int col0 = (bx * a.tile_x - a.c0) & ~1;
         const int row0 = by * a.tile_y - a.c0;
-        const int s = p0 + tk.y;
-        const int e = p0 + tasks[task + 1].y;
+        // this part's points: whole warps of the bin's
+        int s = p0 + tk.y, e = p0 + tasks[task + 1].y;
+        if (a.parts > 1) {
+            const int share = ((e - s + a.parts - 1) / a.parts + 31) & ~31;
+            s += (sub - task * a.parts) * share;
+            e = min(e, s + share);
+            if (s >= e) continue;
+        }
         for (int f0 = a.fa; f0 < a.fa + a.fn; f0 += a.FG) {
             const int fg = min(a.FG, a.fa + a.fn - f0);
             __syncthreads();                   // the tiles of the pass before are consumed
@@ -1159,6 +1167,7 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
     a.fa = p->nwin ? p->win0 : 0;
     a.fn = p->nwin ? p->nwin : a.F;
     a.NG = 1;
+    a.parts = 1;
     a.BW = 0;
     a.box_f = 0;
     // the plan's fitted weight polynomials (fitting them costs the host 10 us at
@@ -1285,6 +1294,13 @@ cudaError_t launch_w(dfsnufft_plan p, void *values) {
             const int passes = (a.fn + a.FG - 1) / a.FG;
             a.FG = (a.fn + passes - 1) / passes;
             const size_t smem_fx = tile * a.FG;
+            // few bins: several CTAs a bin, each staging the tile for whole warps of
+            // its points, until the SMs have a CTA each (64 x 32: 5 of 8 bins hold
+            // points, 20 -> 12 us in 40 CTAs)
+            a.parts = p->num_sms / (p->nbins * M);
+            if (a.parts > 8) a.parts = 8;
+            if (a.parts < 1) a.parts = 1;
+            per = per * a.parts;
             cudaError_t e = dfs_allow_smem((const void *)k_interp_fx<W>, smem_fx);
             if (e) return e;
             return dfs_launch_dependent(

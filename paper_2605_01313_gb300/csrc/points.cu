@@ -232,17 +232,10 @@ __device__ __forceinline__ void block_scan2(int a, int b, int &pa, int &pb, int 
 // rows (the first one in row order, of several), widened by the stencil and
 // rounded out to whole row blocks.  Each thread measures the gaps after its
 // bin rows; the longest wins a shared-memory maximum.
-__device__ void finish_rowrange(const ScanParams &sp, const unsigned char *rows,
-                                unsigned *s_bits, int *s_best, int2 *range_out) {
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
-    const int nb = sp.nbr;
-    if (tid == 0) *s_best = -1;
-    for (int k = wid; k * 32 < nb; k += nw) {
-        const int i = k * 32 + lane;
-        const unsigned b = __ballot_sync(0xffffffffu, i < nb && __ldcg(rows + i) != 0);
-        if (lane == 0) s_bits[k] = b;
-    }
-    __syncthreads();
+__device__ void rowrange_of_bits(const ScanParams &sp, const unsigned *s_bits, int *s_best,
+                                 int2 *range_out) {
+    const int tid = threadIdx.x, nb = sp.nbr;
+    __syncthreads();                           // the bits, and *s_best = -1
     for (int i = tid; i < nb; i += blockDim.x) {
         if (!(s_bits[i >> 5] >> (i & 31) & 1)) continue;
         const int from = i + 1 == nb ? 0 : i + 1;
@@ -265,6 +258,18 @@ __device__ void finish_rowrange(const ScanParams &sp, const unsigned char *rows,
         }
         *range_out = range;
     }
+}
+
+__device__ void finish_rowrange(const ScanParams &sp, const unsigned char *rows,
+                                unsigned *s_bits, int *s_best, int2 *range_out) {
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
+    if (tid == 0) *s_best = -1;
+    for (int k = wid; k * 32 < sp.nbr; k += nw) {
+        const int i = k * 32 + lane;
+        const unsigned b = __ballot_sync(0xffffffffu, i < sp.nbr && __ldcg(rows + i) != 0);
+        if (lane == 0) s_bits[k] = b;
+    }
+    rowrange_of_bits(sp, s_bits, s_best, range_out);
 }
 
 // One chunk's word of the bin scan: 2 flag bits (0 not yet, 1 the chunk's own
@@ -462,6 +467,99 @@ __global__ void __launch_bounds__(256) k_scatter(const FoldRec<R> *__restrict__ 
     pts.store(pos, rec.base, pl, rec.tx, rec.ty);
 }
 
+// set_points of small members in one launch: a CTA a member, its row counts and
+// their prefixes in shared memory, its points (at most SMALL_PPT a thread) in
+// registers between the count and the store.  A step of a few thousand points is
+// a chain of launches of 2 to 4 us each: 64 x 32 in FP64 (2048 points), a
+// counter clear and three kernels of 14 us together before, 9.5 us in this form.
+// Up to SMALL_POINTS points and SMALL_KEYS rows of bins: beyond, one SM's fold
+// costs more than the launches.
+constexpr int SMALL_PPT = 4, SMALL_POINTS = 1024 * SMALL_PPT, SMALL_KEYS = 8192;
+
+template <typename R>
+__global__ void __launch_bounds__(1024) k_points_small(const double *__restrict__ lon,
+                                                       const double *__restrict__ colat,
+                                                       FoldParams f, ScanParams sp,
+                                                       const int *__restrict__ pofs,
+                                                       DfsPoints<R> pts,
+                                                       int2 *__restrict__ task_all,
+                                                       int *__restrict__ n_tasks,
+                                                       int2 *__restrict__ rowrange) {
+    extern __shared__ int s_cnt[];                     // nbins x tile_y row counts
+    __shared__ unsigned s_bits[(DFS_MAX_ROW_BLOCKS + 31) / 32];
+    __shared__ int s_best;
+    const int k = blockIdx.y, tid = threadIdx.x;
+    const int p0 = pofs[k], n = pofs[k + 1] - p0;
+    const int nkeys = sp.nbins * sp.tile_y;
+    for (int i = tid; i < nkeys; i += blockDim.x) s_cnt[i] = 0;
+    if (tid < (DFS_MAX_ROW_BLOCKS + 31) / 32) s_bits[tid] = 0;
+    if (tid == 0) s_best = -1;
+    __syncthreads();
+    int base[SMALL_PPT], key[SMALL_PPT], rank[SMALL_PPT];
+    R ox[SMALL_PPT], oy[SMALL_PPT];
+#pragma unroll
+    for (int u = 0; u < SMALL_PPT; ++u) {
+        const int pl = tid + u * 1024;
+        if (pl >= n) break;
+        int bx, by;
+        unsigned long long tx, ty;
+        const bool ok = fold_point(f, lon[p0 + pl], colat[p0 + pl], bx, by, tx, ty);
+        base[u] = bx | (by << 16);
+        key[u] = rowkey_of(f, bx, by);
+        ox[u] = offset_value<R>(tx, f.odd_w);
+        oy[u] = offset_value<R>(ty, f.odd_w);
+        if (!ok) ox[u] = oy[u] = (R)__int_as_float(0x7fc00000);
+        rank[u] = atomicAdd(&s_cnt[key[u]], 1);
+    }
+    __syncthreads();
+    // each bin's start and its rows' places, the list of non-empty bins
+    int2 *task = task_all + (size_t)k * sp.bstride;
+    int base_s = 0, base_n = 0;
+    for (int b0 = 0; b0 < sp.nbins; b0 += blockDim.x) {
+        const int bin = b0 + tid;
+        int *rc = s_cnt + bin * sp.tile_y;
+        int c = 0;
+        if (bin < sp.nbins)
+            for (int r = 0; r < sp.tile_y; ++r) c += rc[r];
+        int ps, pn, ts, tn;
+        block_scan2(c, c > 0, ps, pn, ts, tn);
+        if (c > 0) {
+            task[base_n + pn] = make_int2(bin, base_s + ps);
+            atomicOr(&s_bits[(bin >> sp.lnbx) >> 5], 1u << ((bin >> sp.lnbx) & 31));
+            int at = base_s + ps;
+            for (int r = 0; r < sp.tile_y; ++r) {
+                const int m = rc[r];
+                rc[r] = at;
+                at += m;
+            }
+        }
+        base_s += ts;
+        base_n += tn;
+    }
+    if (tid == 0) {
+        task[base_n] = make_int2(sp.nbins, base_s);
+        n_tasks[k] = base_n;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < SMALL_PPT; ++u) {
+        const int pl = tid + u * 1024;
+        if (pl >= n) break;
+        pts.store((size_t)p0 + s_cnt[key[u]] + rank[u], base[u], pl, ox[u], oy[u]);
+    }
+    rowrange_of_bits(sp, s_bits, &s_best, rowrange + k);
+}
+
+template <typename R>
+cudaError_t launch_points_small(dfsnufft_plan p, const double *lon, const double *colat,
+                                const FoldParams &f, const ScanParams &sp) {
+    const size_t smem = sizeof(int) * (size_t)sp.nbins * sp.tile_y;     // at most 32 KB
+    k_points_small<R><<<dim3(1, p->n_members), 1024, smem, p->stream>>>(
+        lon, colat, f, sp, p->d_pofs, dfs_points<R>(p), p->d_task_bin, p->d_n_tasks,
+        p->d_rowrange);
+    return cudaGetLastError();
+}
+
 int ilog2(int n) {
     int l = 0;
     while ((1 << l) < n) ++l;
@@ -483,8 +581,6 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
     f.nbx = p->nbx;
     const int M = p->n_members;
     cudaError_t e;
-    if ((e = cudaMemsetAsync(p->d_bin_count, 0, sizeof(int) * (size_t)M * p->cstride, p->stream)))
-        return e;
     const int tpb = 256;
     const dim3 grid((unsigned)((p->max_member_points + tpb - 1) / tpb), M);
     ScanParams sp;
@@ -498,6 +594,12 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
     sp.c0 = p->c0;
     sp.w = q.w;
     sp.n2 = q.n2;
+    if (!p->keep_order && p->max_member_points <= SMALL_POINTS &&
+        p->nbins * q.tile_y <= SMALL_KEYS)
+        return q.dtype == DFSNUFFT_F64 ? launch_points_small<double>(p, lon, colat, f, sp)
+                                       : launch_points_small<float>(p, lon, colat, f, sp);
+    if ((e = cudaMemsetAsync(p->d_bin_count, 0, sizeof(int) * (size_t)M * p->cstride, p->stream)))
+        return e;
     if (p->keep_order) {
         if (q.dtype == DFSNUFFT_F64)
             k_fold_direct<double><<<grid, tpb, 0, p->stream>>>(lon, colat, f, sp, p->d_pofs,
