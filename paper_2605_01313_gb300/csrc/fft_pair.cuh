@@ -114,37 +114,53 @@ __device__ __forceinline__ void pair_butterfly(PairC *v, int t, const float2 *__
     }
 }
 
-template <int LOGN, int LNS, class St, class Hook>
-__device__ __forceinline__ void pair_stages(PairC *v, int t, const float2 *__restrict__ stw,
-                                            PairC *sm, St &st, Hook &after_first_barrier) {
+// Barrier of the T threads of one transform group.  SPLIT: the group has whole
+// warps to itself and waits for its own threads only (hardware barrier id, 1 ..
+// 8), so that the groups of a CTA drift apart, one's exchange under another's
+// butterflies (phi pass, 48 lines: rows of 2048 cells 138 -> 136 us, 1024 36 -> 33
+// us).  The theta pass interleaves its columns in the lanes instead, for the sake
+// of its stores: columns apart (16 bytes of a sector each) 56 -> 66 us.
+template <int T, bool SPLIT>
+__device__ __forceinline__ void group_sync(int id) {
+    if constexpr (!SPLIT) __syncthreads();
+    else if constexpr (T == 32) __syncwarp();
+    else if constexpr (T > 32) asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(T) : "memory");
+    else __syncthreads();
+}
+
+template <int LOGN, int LNS, bool SPLIT, class St, class Hook>
+__device__ __forceinline__ void pair_stages(PairC *v, int t, int id,
+                                            const float2 *__restrict__ stw, PairC *sm, St &st,
+                                            Hook &after_first_barrier) {
     constexpr int E = DFS_FFT_E, LE = 3;
     constexpr int REM = LOGN - LNS;
     if constexpr (REM > 0) {
         constexpr int LR = REM >= LE ? LE : REM;
         constexpr int T = (1 << LOGN) / E;
         if constexpr (LNS > 0) {
-            __syncthreads();
+            group_sync<T, SPLIT>(id);
             if constexpr (LNS == LE) after_first_barrier();
 #pragma unroll
             for (int e = 0; e < E; ++e) v[e] = sm[pair_pad(t + e * T)];
-            if constexpr (REM > LR) __syncthreads();     // the last stage writes no exchange
+            if constexpr (REM > LR) group_sync<T, SPLIT>(id);   // the last stage writes no exchange
         }
         pair_butterfly<(1 << LR), 0, (1 << LNS), stage_table_offset(LOGN, E, LNS), T, REM == LR>(
             v, t, stw, sm, st);
-        pair_stages<LOGN, LNS + LR>(v, t, stw, sm, st, after_first_barrier);
+        pair_stages<LOGN, LNS + LR, SPLIT>(v, t, id, stw, sm, st, after_first_barrier);
     }
 }
 
 // Two length-2^LOGN inverse FFTs (LOGN > 3) of the 2^LOGN / 8 threads t, every
 // thread of the CTA calling: v[e] holds input t + e 2^LOGN / 8 of both, st(i, v)
-// receives output i, stw is the stage-ordered twiddle table of this length.
-// after_first_barrier() runs on every thread when no thread reads the inputs
-// any more; the caller synchronises before it reuses the exchange region.
-template <int LOGN, class St, class Hook>
-__device__ __forceinline__ void pair_fft(const float2 *__restrict__ stw, PairC *sm, int t,
+// receives output i, stw is the stage-ordered twiddle table of this length, id the
+// group's barrier (group_sync).  after_first_barrier() runs on every thread when
+// no thread of its group reads the inputs any more; the caller synchronises before
+// it reuses the exchange region.
+template <int LOGN, bool SPLIT, class St, class Hook>
+__device__ __forceinline__ void pair_fft(const float2 *__restrict__ stw, PairC *sm, int t, int id,
                                          PairC *v, St &st, Hook &after_first_barrier) {
     static_assert(LOGN > 3, "at least two stages");
-    pair_stages<LOGN, 0>(v, t, stw, sm, st, after_first_barrier);
+    pair_stages<LOGN, 0, SPLIT>(v, t, id, stw, sm, st, after_first_barrier);
 }
 
 // Lengths the pair kernels are compiled for.

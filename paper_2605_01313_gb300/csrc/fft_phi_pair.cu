@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(PhiPairCfg<LOGM>::THREADS, PhiPairCfg<LOGM>::M
         dst1[j] = make_float2(re.y, im.y);
     };
     auto none = [] {};
-    pair_fft<LOGM>(stw, sm, t, v, st, none);
+    pair_fft<LOGM, (T >= 32)>(stw, sm, t, c + 1, v, st, none);
 }
 
 template <int LOGM, bool HERM>

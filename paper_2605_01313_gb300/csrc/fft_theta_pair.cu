@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(ThetaPairCfg<LOGH>::THREADS, ThetaPairCfg<LOGH
         auto refill = [&]() {
             if (issuer && nxt < a.total) issue(nxt);
         };
-        pair_fft<LOGH>(stw, sm, t, v, st, refill);
+        pair_fft<LOGH, false>(stw, sm, t, 0, v, st, refill);
         __syncthreads();
     }
 }

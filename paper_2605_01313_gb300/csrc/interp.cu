@@ -833,9 +833,11 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
         return col0 < 0 || col0 + a.BW > a.n1 || row0 < 0 || row0 + TH > a.n2;
     };
     const bool producer = threadIdx.x == blockDim.x - 32;
-    // Claim a sub-task for stage b and start its boxes; false if none is left.
-    auto stage_next = [&](int b) -> bool {
-        int sub = atomicAdd(&wk[0], 1);
+    // Take a sub-task for stage b and start its boxes; false if none is left.  A
+    // CTA's first one is its own index (a thousand claims of one counter at once
+    // took 2 us of a small grid's step), the others are claimed.
+    auto stage_next = [&](int b, bool first) -> bool {
+        int sub = first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(&wk[0], 1);
         if (sub >= total) {
             s_geo[b] = make_int4(0, 0, -1, 0);
             return false;
@@ -864,14 +866,14 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
         return true;
     };
     uint32_t ph0 = 0, ph1 = 0;
-    if (producer) stage_next(0);
+    if (producer) stage_next(0, true);
     __syncthreads();
     for (int it = 0;; ++it) {
         const int cur = it & 1;
         const int4 geo = s_geo[cur];
         if (geo.z < 0) break;
         const int2 fld = s_fld[cur];
-        const bool staged_next = producer && stage_next(cur ^ 1);
+        const bool staged_next = producer && stage_next(cur ^ 1, false);
         // the first point's record, fetched while the boxes land
         const int col0 = geo.x, row0 = geo.y, e = geo.w;
         const int f0 = fld.x, fg = fld.y;
