@@ -24,6 +24,7 @@
 
 #include "df32.cuh"
 #include "fft_core.cuh"
+#include "fft_pair.cuh"
 
 using namespace dfs_fft;
 
@@ -235,6 +236,120 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 1024 : 512) k_fwd_theta(FwdAr
     }
 }
 
+// The FP32 form at compile-time lengths: each thread carries two adjacent
+// columns through the packed transform (fft_pair.cuh), four columns (two groups
+// interleaved in the lanes) a CTA, so that a row of a task is one 32-byte sector
+// in and out; 1024 threads an SM (64 registers each) in several CTAs, which
+// transform at different times.  One input buffer: the next task's rows are
+// requested once every thread has read its inputs.
+// Bound by issue and the shared-memory pipe, like the other packed passes.  The
+// whole step from grid samples, k_fwd_theta<float> (one line a thread, CTAs of
+// 1024 threads) -> this: 64 x 32 (one field) 28.7 -> 26.7 us, 1024 x 512 (three)
+// 105.0 -> 97.5, 2048 x 1024 (one) 151.6 -> 144.5, (three, semi-Lagrangian) 368 ->
+// 355, 4096 x 2048 (three) 1173 -> 1011; 128 x 64 to 512 x 256 within 2 us, none slower.
+template <int LOG>
+__global__ void __launch_bounds__(2 << (LOG - 3), LOG >= 9 ? 1024 >> (LOG - 2) : 8)
+    k_fwd_theta_pair(FwdArgs a, const float2 *__restrict__ spec, const int *__restrict__ parity,
+                     const float2 *__restrict__ tw2, const float2 *__restrict__ stw,
+                     float2 *__restrict__ coef, int nblk, int ntask) {
+    dfs_grid_wait();
+    constexpr int E = DFS_FFT_E, N2 = 1 << LOG, T = N2 / E;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    PairC *ex = reinterpret_cast<PairC *>(smem_raw);
+    float4 *in = reinterpret_cast<float4 *>(ex + 2 * pair_region_stride(N2, 2));  // row: 2 x 16 B
+    const int g = threadIdx.x & 1;                 // column pair
+    const int t = threadIdx.x >> 1;
+    PairC *sm = ex + (size_t)g * pair_region_stride(N2, 2);
+    auto prefetch = [&](int task) {
+        const int f = task / nblk;
+        const int m0 = (task - f * nblk) * 4;
+        const float2 *src = spec + (size_t)f * a.n_lat * a.N1 + m0;
+        for (int q = threadIdx.x; q < 2 * a.n_lat; q += 2 * T)
+            cp_async_16(in + q, src + (size_t)(q >> 1) * a.N1 + 2 * (q & 1));
+    };
+    const float scale = ldexpf(1.f, -(a.log1 + LOG));          // 1 / (N1 N2)
+    const f32x2 sc = pk(scale, scale), msc = pk(-scale, -scale), mone = pk(-1.f, -1.f);
+    const int tw_mask = (N2 << a.tws2) - 1;
+    const int tw_step = 1 << (a.tws2 - 1);
+    const bool aligned = (reinterpret_cast<uintptr_t>(coef) & 15) == 0;
+    if ((int)blockIdx.x < ntask) prefetch(blockIdx.x);
+    for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
+        const int nxt = task + gridDim.x;
+        cp_async_wait_all();
+        __syncthreads();                           // every thread's copies have landed
+        const int f = task / nblk;
+        const int m = (task - f * nblk) * 4 + 2 * g;           // the first column's DFT index
+        const bool ok0 = m <= a.N1 / 2, ok1 = m + 1 <= a.N1 / 2;
+        // the upper half of the doubled column: parity (-1)^m times the mirrored row
+        // (m is even)
+        const float p = parity[f % a.F] < 0 ? -1.f : 1.f;
+        const f32x2 sx = pk(p, -p), sy = pk(-p, p);
+        PairC v[E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = t + e * T;
+            const float4 w = in[2 * (e < E / 2 ? i : N2 - 1 - i) + g];
+            const f32x2 x = pk(w.x, w.z), y = pk(w.y, w.w);
+            // conjugated on input and output: the forward transform
+            v[e] = e < E / 2 ? PairC{x, pmul(y, mone)} : PairC{pmul(x, sx), pmul(y, sy)};
+        }
+        const int mc = m < a.N1 / 2 ? m + a.N1 / 2 : 0;        // centred column
+        float2 *out = coef + (size_t)f * N2 * a.N1 + mc;
+        float2 *mirror = coef + (size_t)f * N2 * a.N1 + (a.N1 - mc);   // column of -m
+        auto st = [&](int k, PairC z) {
+            if (!ok0) return;
+            // mode n = k or k - N2, half-cell phase e^{-i pi n / N2} (see k_fwd_theta)
+            const int n = k < N2 / 2 ? k : k - N2;
+            const PairC u = cmul(z, ldt(&tw2[(n * tw_step) & tw_mask]));
+            const float2 re = unpk(pmul(u.x, sc)), im = unpk(pmul(u.y, msc));
+            float2 *o = out + (size_t)(n + N2 / 2) * a.N1;
+            if (ok1 && aligned) {
+                *reinterpret_cast<float4 *>(o) = make_float4(re.x, im.x, re.y, im.y);
+            } else {
+                o[0] = make_float2(re.x, im.x);
+                if (ok1) o[1] = make_float2(re.y, im.y);
+            }
+            if (n > -N2 / 2) {
+                if (a.full) {
+                    float2 *r = mirror + (size_t)(N2 / 2 - n) * a.N1;
+                    if (m > 0 && m < a.N1 / 2) r[0] = make_float2(re.x, -im.x);
+                    if (m + 1 < a.N1 / 2) r[-1] = make_float2(re.y, -im.y);
+                }
+            } else {
+                if (m > 0 && m < a.N1 / 2) mirror[0] = make_float2(-re.x, im.x);
+                if (m + 1 < a.N1 / 2) mirror[-1] = make_float2(-re.y, im.y);
+            }
+        };
+        auto refill = [&]() {
+            if (nxt < ntask) prefetch(nxt);
+        };
+        pair_fft<LOG, false>(stw, sm, t, 0, v, st, refill);
+        __syncthreads();                           // sm is read before it is refilled
+    }
+}
+
+template <int LOG>
+cudaError_t run_fwd_theta_pair(dfsnufft_plan p, const FwdArgs &a, const void *spec,
+                               const int *d_parity, void *coeffs, int lines) {
+    constexpr int N2 = 1 << LOG;
+    const size_t smem = sizeof(PairC) * 2 * (size_t)pair_region_stride(N2, 2) +
+                        sizeof(float2) * 4 * (size_t)a.n_lat;
+    auto kern = k_fwd_theta_pair<LOG>;
+    cudaError_t e = allow_smem(kern, smem);
+    if (e) return e;
+    const int nblk = (a.N1 / 2 + 1 + 3) / 4;
+    const int ntask = nblk * lines;
+    int occ = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, N2 / 4, smem) != cudaSuccess ||
+        occ < 1)
+        occ = 1;
+    const long long want = (long long)p->num_sms * occ;
+    return dfs_launch_dependent(kern, dim3((unsigned)(want < ntask ? want : ntask)),
+                                dim3(N2 / 4), smem, p->stream, a, (const float2 *)spec, d_parity,
+                                (const float2 *)p->d_tw2, (const float2 *)p->d_stw_theta,
+                                (float2 *)coeffs, nblk, ntask);
+}
+
 // The plan's tables for the pass's arithmetic: twiddles of lengths n1 and n2
 // and the stage-ordered table of length n1/2 (double-single copies for df32).
 template <typename R> struct FwdTables {
@@ -348,11 +463,26 @@ cudaError_t launch_forward(dfsnufft_plan p, const void *samples, const int *d_pa
         default: e = run_fwd_phi<R, 0>(p, a, samples, spec, lines, nullptr, nullptr, emax); break;
     }
     if (e) return e;
-    switch (ct2 ? a.log2 : 0) {
-        case 9: return run_fwd_theta<R, 9>(p, a, spec, d_parity, coeffs, lines, emax);
-        case 10: return run_fwd_theta<R, 10>(p, a, spec, d_parity, coeffs, lines, emax);
-        case 11: return run_fwd_theta<R, 11>(p, a, spec, d_parity, coeffs, lines, emax);
-        default: return run_fwd_theta<R, 0>(p, a, spec, d_parity, coeffs, lines, emax);
+    if constexpr (std::is_same<R, float>::value) {
+        // the packed form wherever its table fits; k_fwd_theta for N2 of 16 and 32 and
+        // fine grids of other ratios
+        switch (tb.stw_half && q.n2 == 2 * q.N2 ? a.log2 : 0) {
+            case 6: return run_fwd_theta_pair<6>(p, a, spec, d_parity, coeffs, lines);
+            case 7: return run_fwd_theta_pair<7>(p, a, spec, d_parity, coeffs, lines);
+            case 8: return run_fwd_theta_pair<8>(p, a, spec, d_parity, coeffs, lines);
+            case 9: return run_fwd_theta_pair<9>(p, a, spec, d_parity, coeffs, lines);
+            case 10: return run_fwd_theta_pair<10>(p, a, spec, d_parity, coeffs, lines);
+            case 11: return run_fwd_theta_pair<11>(p, a, spec, d_parity, coeffs, lines);
+            case 12: return run_fwd_theta_pair<12>(p, a, spec, d_parity, coeffs, lines);
+            default: return run_fwd_theta<R, 0>(p, a, spec, d_parity, coeffs, lines);
+        }
+    } else {
+        switch (ct2 ? a.log2 : 0) {
+            case 9: return run_fwd_theta<R, 9>(p, a, spec, d_parity, coeffs, lines, emax);
+            case 10: return run_fwd_theta<R, 10>(p, a, spec, d_parity, coeffs, lines, emax);
+            case 11: return run_fwd_theta<R, 11>(p, a, spec, d_parity, coeffs, lines, emax);
+            default: return run_fwd_theta<R, 0>(p, a, spec, d_parity, coeffs, lines, emax);
+        }
     }
 }
 
