@@ -365,8 +365,7 @@ template <typename R> struct FwdTables {
 
 template <typename R, int LOG>
 cudaError_t run_fwd_phi(dfsnufft_plan p, const FwdArgs &a, const void *samples, void *spec,
-                        int lines, const int *d_parity = nullptr, void *g1 = nullptr,
-                        const int *emax = nullptr) {
+                        int lines, const int *d_parity, void *g1, const int *emax) {
     typedef typename CxT<R>::type C;
     typedef typename FwdIO<R>::In In;
     constexpr int E = DFS_FFT_E;
@@ -389,6 +388,32 @@ cudaError_t run_fwd_phi(dfsnufft_plan p, const FwdArgs &a, const void *samples, 
             nullptr, nullptr, emax);
     }
     return cudaGetLastError();
+}
+
+// The longitude pass at its length.  The plan's stage-ordered table is for length
+// n1/2: it serves the compile-time lengths when the fine grid is twice the modes.
+// FP32 has all of 64 .. 4096 (runtime length -> compile-time, the step from grid
+// samples: 4096 x 2048 1015 -> 950 us, 256 x 128 44.1 -> 42.5, 128 x 64 40.8 -> 39.7,
+// 64 x 32 26.7 -> 26.0), the others the lengths of medium and large grids.
+template <typename R>
+cudaError_t launch_fwd_phi(dfsnufft_plan p, const FwdArgs &a, const void *samples, void *spec,
+                           int lines, const int *d_parity, void *g1, const int *emax) {
+    const FwdTables<R> tb(p);
+    const int log = tb.stw_phi && p->prm.n1 == 2 * a.N1 ? a.log1 : 0;
+    if constexpr (std::is_same<R, float>::value) {
+        switch (log) {
+            case 6: return run_fwd_phi<R, 6>(p, a, samples, spec, lines, d_parity, g1, emax);
+            case 7: return run_fwd_phi<R, 7>(p, a, samples, spec, lines, d_parity, g1, emax);
+            case 8: return run_fwd_phi<R, 8>(p, a, samples, spec, lines, d_parity, g1, emax);
+            case 12: return run_fwd_phi<R, 12>(p, a, samples, spec, lines, d_parity, g1, emax);
+        }
+    }
+    switch (log) {
+        case 9: return run_fwd_phi<R, 9>(p, a, samples, spec, lines, d_parity, g1, emax);
+        case 10: return run_fwd_phi<R, 10>(p, a, samples, spec, lines, d_parity, g1, emax);
+        case 11: return run_fwd_phi<R, 11>(p, a, samples, spec, lines, d_parity, g1, emax);
+        default: return run_fwd_phi<R, 0>(p, a, samples, spec, lines, d_parity, g1, emax);
+    }
 }
 
 template <typename R, int LOG>
@@ -444,9 +469,8 @@ cudaError_t launch_forward(dfsnufft_plan p, const void *samples, const int *d_pa
     const int lines = p->n_members * p->n_fields;
     constexpr bool df = std::is_same<R, df32>::value;
     const FwdTables<R> tb(p);
-    // the plan's stage-ordered tables are for lengths n1/2 and n2/2: they serve
-    // the compile-time drivers when the fine grid is twice the modes
-    const bool ct1 = tb.stw_phi && q.n1 == 2 * q.N1 && a.log1 >= 9 && a.log1 <= 11;
+    // the plan's stage-ordered table is for length n2/2: it serves the compile-time
+    // drivers when the fine grid is twice the modes
     const bool ct2 = tb.stw_half && q.n2 == 2 * q.N2 && a.log2 >= 9 && a.log2 <= 11;
     cudaError_t e;
     const int *emax = nullptr;
@@ -456,12 +480,7 @@ cudaError_t launch_forward(dfsnufft_plan p, const void *samples, const int *d_pa
         if (e) return e;
         emax = p->d_emax;
     }
-    switch (ct1 ? a.log1 : 0) {
-        case 9: e = run_fwd_phi<R, 9>(p, a, samples, spec, lines, nullptr, nullptr, emax); break;
-        case 10: e = run_fwd_phi<R, 10>(p, a, samples, spec, lines, nullptr, nullptr, emax); break;
-        case 11: e = run_fwd_phi<R, 11>(p, a, samples, spec, lines, nullptr, nullptr, emax); break;
-        default: e = run_fwd_phi<R, 0>(p, a, samples, spec, lines, nullptr, nullptr, emax); break;
-    }
+    e = launch_fwd_phi<R>(p, a, samples, spec, lines, nullptr, nullptr, emax);
     if (e) return e;
     if constexpr (std::is_same<R, float>::value) {
         // the packed form wherever its table fits; k_fwd_theta for N2 of 16 and 32 and
@@ -525,13 +544,7 @@ static cudaError_t launch_fwd_phi_gl(dfsnufft_plan p, const void *samples, const
     a.K = K;
     a.gpitch = pitch;
     const int lines = p->n_members * p->n_fields;
-    const bool ct1 = p->d_stw_phi && q.n1 == 2 * q.N1 && a.log1 >= 9 && a.log1 <= 11;
-    switch (ct1 ? a.log1 : 0) {
-        case 9: return run_fwd_phi<R, 9>(p, a, samples, g0, lines, d_parity, g1);
-        case 10: return run_fwd_phi<R, 10>(p, a, samples, g0, lines, d_parity, g1);
-        case 11: return run_fwd_phi<R, 11>(p, a, samples, g0, lines, d_parity, g1);
-        default: return run_fwd_phi<R, 0>(p, a, samples, g0, lines, d_parity, g1);
-    }
+    return launch_fwd_phi<R>(p, a, samples, g0, lines, d_parity, g1, nullptr);
 }
 
 cudaError_t dfs_launch_fwd_phi_gl(dfsnufft_plan p, const void *samples, const int *d_parity,

@@ -1,5 +1,5 @@
-"""The packed FP32 colatitude pass of the grid-to-coefficients transform at all
-lengths it is compiled for (64 .. 4096 doubled rows) and just below, against the
+"""The FP32 passes of the grid-to-coefficients transform at all lengths they are
+compiled for (64 .. 4096 in each direction) and just below, against the
 oracle's doubled-torus sums: the fewest columns (blocks with one column in use),
 odd numbers of fields, members, both parities, outputs that are 8-byte but not
 16-byte aligned, and the half spectrum that real-field plans interpolate from.
@@ -35,7 +35,8 @@ def plan_for(n_lon, n_lat, F, members=1, real=True):
 @pytest.mark.parametrize("n_lon,n_lat,members", [(16, 16, 1), (16, 32, 3), (64, 64, 1),
                                                  (16, 128, 1), (16, 256, 2), (32, 512, 1),
                                                  (64, 512, 3), (16, 1024, 1), (64, 1024, 2),
-                                                 (16, 2048, 1)])
+                                                 (16, 2048, 1), (64, 8, 1),
+                                                 (128, 16, 2), (256, 8, 1), (4096, 8, 1)])
 def test_coefficients(torch_cuda, n_lon, n_lat, members, aligned):
     torch = torch_cuda
     rng = np.random.default_rng(n_lon + n_lat + members)
