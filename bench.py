@@ -256,10 +256,12 @@ def interp_flops(prm, n_fields, n_points):
 
 
 def df32_interp_ops(prm, n_fields, n_points):
-    """FP32 arithmetic instructions (FADD, FMUL, FFMA: one each) of one
-    double-single interpolation launch (FP64 plans, k_interp_df), counted from
-    its operations: TwoSum 6, TwoProduct 2, a double-single product 7 (with its
-    fast renormalisation), sum 11, Horner step 15, Dot2 step 12.  Per point: the
+    """FP32 arithmetic instructions (FADD, FMUL, FFMA: one each) of one FP64
+    interpolation launch in compensated double-single arithmetic, a fixed measure
+    of its work (the kernel, k_interp_fx, sums in fixed point and needs about a
+    third fewer instructions), counted from its operations: TwoSum 6, TwoProduct 2,
+    a double-single product 7 (with its fast renormalisation), sum 11, Horner step
+    15, Dot2 step (one compensated multiply-add) 12.  Per point: the
     x and y weights, each (w + 1) / 2 mirror pairs of an even and an odd Horner
     chain (w - 1 steps together), one product s o and the two sums, plus u = s^2
     for each axis; per point and field, w stencil rows of w Dot2 steps, each row
@@ -577,9 +579,9 @@ def measure(args, name, wl, ws, rank, dev, serving, cpu_seconds=None):
               key=lambda k: per_stage_ms[k] or 0.0)
     dom_ms = per_stage_ms[dom]
     if wl.dtype == "f64" and dom == "interp" and not (prm["flags"] & 2):
-        # FP64 plans interpolate in double-single arithmetic on the FP32 units:
-        # the stage's FP32 instructions (df32_interp_ops) against the FP32 pipe's
-        # instruction rate, measured live by the FMA probe (FLOP/s / 2)
+        # FP64 plans interpolate on the FP32 and integer units: the stage's work as
+        # FP32 instructions (df32_interp_ops) against the FP32 pipe's instruction
+        # rate, measured live by the FMA probe (FLOP/s / 2)
         fma32 = nufft.dfsnufft_probe_fma_rate("f32", 20.0)
         ops = df32_interp_ops(prm, F, P)
         achieved = ops / (dom_ms * 1e-3) / 1e12

@@ -242,11 +242,12 @@ __global__ void __launch_bounds__(sizeof(R) == 4 ? 1024 : 512) k_fwd_theta(FwdAr
 // in and out; 1024 threads an SM (64 registers each) in several CTAs, which
 // transform at different times.  One input buffer: the next task's rows are
 // requested once every thread has read its inputs.
-// Bound by issue and the shared-memory pipe, like the other packed passes.  The
-// whole step from grid samples, k_fwd_theta<float> (one line a thread, CTAs of
-// 1024 threads) -> this: 64 x 32 (one field) 28.7 -> 26.7 us, 1024 x 512 (three)
-// 105.0 -> 97.5, 2048 x 1024 (one) 151.6 -> 144.5, (three, semi-Lagrangian) 368 ->
-// 355, 4096 x 2048 (three) 1173 -> 1011; 128 x 64 to 512 x 256 within 2 us, none slower.
+// Bound by the load/store pipe (68%) and the latency of the table loads.  2048 x
+// 1024, three fields: k_fwd_theta<float> (one line a thread, CTAs of 1024 threads)
+// 47 us -> 35 (algorithmic bytes 75 MB).  The whole step from grid samples: 64 x 32
+// (one field) 28.7 -> 26.7 us, 1024 x 512 (three) 105.0 -> 97.5, 2048 x 1024 (one)
+// 151.6 -> 144.5, (three, semi-Lagrangian) 368 -> 355, 4096 x 2048 (three) 1173 ->
+// 1011; 128 x 64 to 512 x 256 within 2 us, none slower.
 template <int LOG>
 __global__ void __launch_bounds__(2 << (LOG - 3), LOG >= 9 ? 1024 >> (LOG - 2) : 8)
     k_fwd_theta_pair(FwdArgs a, const float2 *__restrict__ spec, const int *__restrict__ parity,
