@@ -79,7 +79,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
             if (threadIdx.x == 0) emax[f] = em;             // every CTA writes the same
             const int sl = df_line_shift(em);
             for (int i = t; i < a.tcols; i += T) {
-                const int d = df_line_shift(ce[i]) - sl;    // at most 0 for finite lines
+                // at most 0 for finite lines; ce = 0 is a column of zeros
+                const int d = df_line_shift(ce[i]) - sl;
                 const float k = em >= 0x7ff ? 1.f
                                 : ce[i] == 0 || d < -126 ? 0.f
                                                          : __int_as_float((127 + d) << 23);

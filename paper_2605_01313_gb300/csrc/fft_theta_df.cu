@@ -50,9 +50,15 @@ template <int LOGN> struct ThetaDfCfg {
     static constexpr int MINB = 1024 / THREADS > 16 ? 16 : 1024 / THREADS;
 };
 
-__device__ __forceinline__ int exp_of(double2 v) {
-    return max(((int)__double2hiint(v.x) >> 20) & 0x7ff, ((int)__double2hiint(v.y) >> 20) & 0x7ff);
+// Biased exponent for the column scale.  A subnormal number counts as exponent 1
+// (scale 2^1022), so that a column of them keeps its digits beside the line's
+// other columns; 0 is left for zeros.
+__device__ __forceinline__ int exp_of(double v) {
+    const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+    const int e = (int)(h >> 20);
+    return e ? e : (h | (unsigned)__double2loint(v)) != 0;
 }
+__device__ __forceinline__ int exp_of(double2 v) { return max(exp_of(v.x), exp_of(v.y)); }
 
 template <int LOGN, bool HERM>
 __global__ void __launch_bounds__(ThetaDfCfg<LOGN>::THREADS, ThetaDfCfg<LOGN>::MINB)
