@@ -71,7 +71,9 @@ __global__ void __launch_bounds__(MAXT, MINB)
             if (threadIdx.x == 0) s_emax = 0;
             int m = 0;
             for (int i = threadIdx.x; i < a.tcols; i += blockDim.x) m = max(m, ce[i]);
-            m = __reduce_max_sync(__activemask(), m);
+            // every thread of the warp is named (a CTA may have 8 or 16 threads), so the
+            // lanes that took one column more join the others here
+            m = __reduce_max_sync(blockDim.x >= 32 ? 0xffffffffu : (1u << blockDim.x) - 1, m);
             __syncthreads();
             if ((threadIdx.x & 31) == 0) atomicMax(&s_emax, m);
             __syncthreads();

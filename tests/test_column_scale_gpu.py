@@ -4,8 +4,8 @@ at full accuracy whatever the others hold, down to subnormal numbers.
 
 Reference: the FP64 oracle on the coefficients times 2^k, a power of two that
 makes them normal numbers (exact, also for subnormal ones); the values times 2^k
-are exact too.  Tolerance: 1e-11 of the largest value, the bound of every FP64
-test at 1e-12."""
+are exact too.  Tolerance: 10 x the requested accuracy of the largest value, as
+in every FP64 test (1e-11 at 1e-12)."""
 import math
 
 import numpy as np
@@ -17,9 +17,6 @@ from test_fft_pair_gpu import mirror_substituted
 
 pytestmark = pytest.mark.gpu
 
-BOUND = 1e-11
-
-
 @pytest.fixture(scope="module")
 def torch_cuda():
     import torch
@@ -29,14 +26,14 @@ def torch_cuda():
     return torch
 
 
-def check(torch, c, real, k=0):
+def check(torch, c, real, k=0, tol=1e-12):
     """Every field of c against the oracle, both times 2^k."""
     from paper_2605_01313_gb300 import Plan
     from paper_2605_01313_gb300.nufft import Options
     rng = np.random.default_rng(5)
     F, N2, N1 = c.shape
     lon, colat = rng.uniform(-1.0, 7.0, 150), rng.uniform(0.0, math.pi, 150)
-    with Plan(N1, N2 // 2, 1e-12, "f64", F, options=Options.make(real_fields=real)) as plan:
+    with Plan(N1, N2 // 2, tol, "f64", F, options=Options.make(real_fields=real)) as plan:
         plan.set_points(torch.from_numpy(lon).cuda(), torch.from_numpy(colat).cuda())
         vals = plan.execute(torch.from_numpy(c).cuda())
         plan.check()
@@ -44,7 +41,7 @@ def check(torch, c, real, k=0):
     up = np.ldexp(c.real, k) + 1j * np.ldexp(c.imag, k)
     ref = oracle.evaluate(mirror_substituted(up) if real else up, lon, colat)
     for f in range(F):
-        assert oracle.rel_linf(vals[f], ref[f].real) <= BOUND, f
+        assert oracle.rel_linf(vals[f], ref[f].real) <= 10 * tol, f
 
 
 def noise(rng, F, n_lon, n_lat):
@@ -89,3 +86,16 @@ def test_largest_column_anywhere(torch_cuda, factor, real):
         if real and 0 < q < n_lon // 2:  # the column a real-field plan reads in its place
             c[q, :, n_lon - q] /= factor
     check(torch_cuda, c, real)
+
+
+# the same at narrow rows and kernels, where the phi pass runs CTAs of less than a warp
+@pytest.mark.parametrize("real", [True, False])
+@pytest.mark.parametrize("n_lon", [4, 6, 8])
+def test_largest_column_in_part_warps(torch_cuda, n_lon, real):
+    rng = np.random.default_rng(84)
+    c = noise(rng, n_lon, n_lon, 16) * 2.0 ** -20
+    for q in range(n_lon):
+        c[q, :, q] *= 2.0 ** 20
+        if real and 0 < q < n_lon // 2:
+            c[q, :, n_lon - q] *= 2.0 ** 20
+    check(torch_cuda, c, real, tol=1e-4)
