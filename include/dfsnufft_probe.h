@@ -7,6 +7,8 @@
 #ifndef DFSNUFFT_PROBE_H
 #define DFSNUFFT_PROBE_H
 
+#include <stdint.h>
+
 #ifdef __cplusplus
 extern "C" {
 #endif
@@ -40,6 +42,18 @@ int dfsnufft_selftest_wait_timeout(long long cycles, int *device_status, double 
  * dfsnufft_ensemble_run computes normally.  DFSNUFFT_ERR_NO_POINTS if the
  * ensemble is not in persistent mode or has not run a step yet. */
 int dfsnufft_ensemble_selftest_queue_timeout(struct dfsnufft_ensemble_s *ens, long long cycles);
+
+/* Self-test of the bin scan's waits: set_points (n_points[members], lon, colat as
+ * for dfsnufft_set_points_batch) whose first chunk of 512 bins never publishes its
+ * totals, so that the chunks after it wait in vain.  Each wait gives up after
+ * `cycles` SM clock cycles (1 <= cycles <= 4e9).  Synchronous.  Returns
+ * DFSNUFFT_ERR_TIMEOUT (the expected outcome) or DFSNUFFT_OK, without making the
+ * failure sticky: until the next set_points, execute evaluates nothing and writes
+ * NaN.  DFSNUFFT_ERR_UNSUPPORTED for plans whose points are not sorted by the
+ * scan (at most 512 bins, DFSNUFFT_KEEP_ORDER). */
+int dfsnufft_plan_selftest_scan_timeout(struct dfsnufft_plan_s *plan, const int64_t *n_points,
+                                        const double *lon, const double *colat,
+                                        long long cycles);
 
 #ifdef __cplusplus
 }

@@ -86,6 +86,7 @@ struct dfsnufft_plan_s {
     int bstride;            // per-member stride of the bin arrays: >= nbins + 1, multiple of 4
     int cstride;            // per-member stride of d_bin_count (dfs_cstride)
     int nch;                // bin-scan chunks, ceil(nbins / DFS_SCAN_CHUNK)
+    long long scan_budget;  // self-test of the scan's wait: its limit in SM cycles, else 0
     cudaStream_t stream;
 
     // device buffers owned by the plan
@@ -101,7 +102,7 @@ struct dfsnufft_plan_s {
     int *d_bin_start;       // members x bstride (nbins + 1 used), member-local positions
     int2 *d_task_bin;       // members x bstride: the non-empty bins in order, (bin, its
                             // start), then (nbins, the member's points)
-    int *d_n_tasks;         // members
+    int *d_n_tasks;         // members; -1: the bin scan gave up, the lists are not valid
     int2 *d_rowrange;           // per member: circular range of needed fine rows (first, count)
     int *d_pofs;                // members + 1 point offsets (device)
     int64_t *h_pofs;            // members + 1 point offsets of the current points (host)

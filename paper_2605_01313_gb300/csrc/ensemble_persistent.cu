@@ -220,6 +220,12 @@ __device__ void interp_task(const EnsGroup &g, int member, int slot0, unsigned c
     const int ntask = g.n_tasks[member];
     const int2 *tasks = g.task_bin + (size_t)member * g.bstride;
     const float *hc = g.horner;
+    if (ntask < 0) {                            // the bin scan gave up (points.cu)
+        if (slot0 == 0)
+            for (int i = threadIdx.x; i < g.F * Pk; i += kThreads)
+                g.values[(size_t)g.F * p0 + i] = __int_as_float(0x7fc00000);
+        return;
+    }
     for (int slot = slot0; slot < slot0 + ENS_BINS && slot < ntask; ++slot) {
         const int bin = tasks[slot].x;
         const int by = bin / g.nbx;

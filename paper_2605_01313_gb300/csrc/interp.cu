@@ -46,6 +46,17 @@ struct InterpArgs {
 __device__ __forceinline__ int cell_x(int cell) { return cell & 0xffff; }
 __device__ __forceinline__ int cell_y(int cell) { return cell >> 16; }
 
+// A member whose bin scan gave up (n_tasks = -1, points.cu): no list to walk, and
+// its n values at `out` become NaN.
+template <typename R>
+__device__ __forceinline__ bool points_invalid(int ntask, R *out, size_t n) {
+    if (ntask >= 0) return false;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+         i += (size_t)gridDim.x * blockDim.x)
+        out[i] = (R)__int_as_float(0x7fc00000);
+    return true;
+}
+
 // Kernel weights by Horner's rule: for tap a the weight phi((a - c0) - t) is a
 // degree-W polynomial in s = t - mid (mid = 0 for odd W, 1/2 for even W),
 // fitted on the host (dfsnufft_es_horner) to about e^-beta, the size of the
@@ -100,6 +111,8 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
+    if (points_invalid(ntask, out_all + (size_t)a.F * p0 + (size_t)a.fa * Pk, (size_t)a.fn * Pk))
+        return;
     const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
         const int2 tk = tasks[task];
@@ -303,6 +316,8 @@ __global__ void __launch_bounds__(256, 2) k_interp_fx(InterpArgs a,
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
+    if (points_invalid(ntask, out_all + (size_t)a.F * p0 + (size_t)a.fa * Pk, (size_t)a.fn * Pk))
+        return;
     const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int sub = blockIdx.x; sub < ntask * a.parts; sub += gridDim.x) {
         const int task = sub / a.parts;
@@ -690,6 +705,8 @@ __global__ void __launch_bounds__(128) k_interp_f32(InterpArgs a,
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
     const int ntask = n_tasks[k];
+    if (points_invalid(ntask, out_all + (size_t)a.F * p0 + (size_t)a.fa * Pk, (size_t)a.fn * Pk))
+        return;
     const int2 *tasks = task_all + (size_t)k * a.bstride;
     for (int task = blockIdx.x; task < ntask; task += gridDim.x) {
         const int2 tk = tasks[task];
@@ -819,7 +836,9 @@ __global__ void __launch_bounds__(128) k_interp_tma(InterpArgs a,
     const int k = blockIdx.y;
     const int p0 = pofs[k];
     const int Pk = pofs[k + 1] - p0;
-    const int total = n_tasks[k] * a.NG;
+    const int ntask = n_tasks[k], total = ntask * a.NG;
+    if (points_invalid(ntask, out_all + (size_t)a.F * p0 + (size_t)a.fa * Pk, (size_t)a.fn * Pk))
+        return;
     const int2 *tasks = task_all + (size_t)k * a.bstride;
     int *wk = work + 2 * k;
     if (threadIdx.x == 0) {

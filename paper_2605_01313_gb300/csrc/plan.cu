@@ -8,6 +8,7 @@
 #include <new>
 
 #include "common.cuh"
+#include "dfsnufft_probe.h"
 #include "fft_core.cuh"
 
 #define DFS_VERSION "dfsnufft 0.1 (sm_103a)"
@@ -755,6 +756,23 @@ extern "C" int dfsnufft_set_points_batch(dfsnufft_plan p, const int64_t *n_point
     return DFSNUFFT_OK;
 }
 
+extern "C" int dfsnufft_plan_selftest_scan_timeout(dfsnufft_plan p, const int64_t *n_points,
+                                                   const double *lon, const double *colat,
+                                                   long long cycles) {
+    if (!p || cycles < 1 || cycles > 4000000000LL) return DFSNUFFT_ERR_INVALID_ARG;
+    if (p->status) return p->status;
+    if (p->keep_order || p->nch < 2) return DFSNUFFT_ERR_UNSUPPORTED;
+    p->scan_budget = cycles;
+    const int rc = dfsnufft_set_points_batch(p, n_points, lon, colat);
+    p->scan_budget = 0;
+    if (rc) return rc;
+    DFS_CK(p, cudaStreamSynchronize(p->stream));
+    int st = 0;
+    DFS_CK(p, cudaMemcpy(&st, p->d_status, sizeof(int), cudaMemcpyDeviceToHost));
+    DFS_CK(p, cudaMemset(p->d_status, 0, sizeof(int)));
+    return st ? DFSNUFFT_ERR_TIMEOUT : DFSNUFFT_OK;
+}
+
 extern "C" int dfsnufft_set_points(dfsnufft_plan p, int64_t n_points, const double *lon,
                                    const double *colat) {
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
@@ -1220,7 +1238,7 @@ extern "C" int dfsnufft_plan_point_stats(dfsnufft_plan p, int64_t *rows_needed,
     int64_t rows = 0, bins = 0;
     for (int k = 0; k < M; ++k) {
         rows += range[k].y;
-        bins += ntask[k];
+        bins += ntask[k] > 0 ? ntask[k] : 0;
     }
     free(range);
     free(ntask);

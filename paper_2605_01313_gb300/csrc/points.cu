@@ -166,13 +166,16 @@ struct ScanParams {
     int cstride;              // per-member stride of the count slice (scan workspace + counts)
     int nch;                  // chunks of DFS_SCAN_CHUNK bins
     int tile_y, c0, w, n2;
+    long long budget;         // SM cycles the look-back waits at most
+    int mute;                 // self-test: chunk 0 publishes nothing
 };
 
 // Layout of a member's count slice (cstride ints, zeroed before each
-// set_points): the scan's ticket and completion counters, the bin-row flags
-// (bytes), one 64-bit word a chunk, then the row counts.
+// set_points): the scan's ticket and completion counters and its failure flag, the
+// bin-row flags (bytes), one 64-bit word a chunk, then the row counts.
 __device__ __forceinline__ int *ws_ticket(int *slice) { return slice; }
 __device__ __forceinline__ int *ws_done(int *slice) { return slice + 1; }
+__device__ __forceinline__ int *ws_failed(int *slice) { return slice + 2; }
 __device__ __forceinline__ unsigned char *ws_rows(int *slice) {
     return reinterpret_cast<unsigned char *>(slice + 4);
 }
@@ -273,7 +276,8 @@ __device__ void finish_rowrange(const ScanParams &sp, const unsigned char *rows,
 }
 
 // One chunk's word of the bin scan: 2 flag bits (0 not yet, 1 the chunk's own
-// totals, 2 the totals through it), 31 bits of non-empty bins, 31 of points.
+// totals, 2 the totals through it, 3 the chunk gave up), 31 bits of non-empty
+// bins, 31 of points.
 __device__ __forceinline__ unsigned long long chunk_word(int flag, int ne, int sum) {
     return ((unsigned long long)flag << 62) | ((unsigned long long)ne << 31) |
            (unsigned long long)sum;
@@ -282,13 +286,19 @@ __device__ __forceinline__ unsigned long long chunk_word(int flag, int ne, int s
 // The bin scan in one pass.  grid (nch, members), a thread a bin: the exclusive
 // prefix of the bin's row counts (in place: the offset of each row inside the
 // bin), its start, the list of non-empty bins in bin order and the bin-row
-// flags.  A chunk's offsets come from the chunks before it by looking back:
-// each publishes its own totals, then the totals through it, and warp 0 reads
-// 32 words at a time until it meets one of the latter.  Chunks are taken by
-// ticket, so every word waited for belongs to a CTA that is already running;
-// the wait is bounded (about a second, then DFS_STATUS_TIMEOUT, with offsets that
-// stay inside the member's slice: they are sums of fewer counts).  The last CTA
-// of a member to finish finds the needed row range.
+// flags.  A chunk's offsets come from the chunks before it by looking back
+// (decoupled look-back, Merrill and Garland 2016): each publishes its own totals,
+// then the totals through it, and warp 0 reads 32 words at a time until it meets
+// one of the latter.  Chunks are taken by ticket, so every word waited for belongs
+// to a CTA that is already running.  The last CTA of a member to finish finds the
+// needed row range.
+//
+// The wait is bounded (DFS_WAIT_CYCLES, about a second).  A chunk that gives up
+// sets DFS_STATUS_TIMEOUT and the member's failure flag and tells the chunks after
+// it; its starts are sums of fewer counts, so the scatter stays inside the
+// member's slice, but the list and the records have gaps.  The last CTA then
+// leaves n_tasks = -1 and an empty row range, whatever the chunks stored: no pass
+// reads the list or the records, and the interpolation writes NaN.
 //
 // Bound by latency: a chain of a ticket, the row counts, two block scans and the
 // words before it.  One kernel in place of a row prefix, chunk sums and a second
@@ -348,7 +358,8 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     block_scan2(c, c > 0, ps, pn, ts, tn);
     if (tid < 32) {
         int bs = 0, bn = 0;
-        if (tid == 0)
+        bool failed = false;
+        if (tid == 0 && !(sp.mute && chunk == 0))
             *(volatile unsigned long long *)&words[chunk] = chunk_word(chunk ? 1 : 2, tn, ts);
         const long long t0 = clock64();
         for (int base = chunk - 1; base >= 0; base -= 32) {
@@ -357,12 +368,11 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
             bool late = false;
             if (idx >= 0) {
                 volatile unsigned long long *p = &words[idx];
-                while (((w = *p) >> 62) == 0 && !late) late = clock64() - t0 > DFS_WAIT_CYCLES;
+                while (((w = *p) >> 62) == 0 && !late) late = clock64() - t0 > sp.budget;
+                late |= (w >> 62) == 3;
             }
-            if (__any_sync(0xffffffffu, late)) {
-                if (tid == 0 && status) atomicExch(status, DFS_STATUS_TIMEOUT);
-                break;
-            }
+            failed = __any_sync(0xffffffffu, late);
+            if (failed) break;
             const unsigned through = __ballot_sync(0xffffffffu, (w >> 62) == 2);
             const bool use = !through || tid <= __ffs(through) - 1;
             bs += __reduce_add_sync(0xffffffffu, use ? (int)(w & 0x7fffffff) : 0);
@@ -370,8 +380,13 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
             if (through) break;
         }
         if (tid == 0) {
+            if (failed) {
+                if (status) atomicExch(status, DFS_STATUS_TIMEOUT);
+                atomicExch(ws_failed(slice), 1);
+            }
             if (chunk)
-                *(volatile unsigned long long *)&words[chunk] = chunk_word(2, bn + tn, bs + ts);
+                *(volatile unsigned long long *)&words[chunk] =
+                    chunk_word(failed ? 3 : 2, bn + tn, bs + ts);
             s_pre[0] = bs;
             s_pre[1] = bn;
         }
@@ -398,6 +413,10 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     if (!s_last) return;
     __threadfence();
     finish_rowrange(sp, rows, s_bits, &s_best, rowrange + member);
+    if (tid == 0 && __ldcg(ws_failed(slice))) {
+        n_tasks[member] = -1;
+        rowrange[member] = make_int2(0, 0);
+    }
 }
 
 // Points kept in the caller's order (DFSNUFFT_KEEP_ORDER): fold every point to
@@ -594,6 +613,8 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
     sp.c0 = p->c0;
     sp.w = q.w;
     sp.n2 = q.n2;
+    sp.budget = p->scan_budget ? p->scan_budget : DFS_WAIT_CYCLES;
+    sp.mute = p->scan_budget != 0;
     if (!p->keep_order && p->max_member_points <= SMALL_POINTS &&
         p->nbins * q.tile_y <= SMALL_KEYS)
         return q.dtype == DFSNUFFT_F64 ? launch_points_small<double>(p, lon, colat, f, sp)

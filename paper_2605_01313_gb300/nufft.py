@@ -47,6 +47,7 @@ EXPORTS = (
     "dfsnufft_departure_points", "dfsnufft_rotate_to_arrival", "dfsnufft_lagrange_interp",
     "dfsnufft_plan_latitudes", "dfsnufft_plan_host_copy_bytes",
     "dfsnufft_ensemble_set_persistent", "dfsnufft_ensemble_selftest_queue_timeout",
+    "dfsnufft_plan_selftest_scan_timeout",
 )
 REAL_FIELDS = 1
 KEEP_ORDER = 2
@@ -173,6 +174,7 @@ def lib():
         L.dfsnufft_server_wait.argtypes = [vp, i64, f64, ctypes.POINTER(i32), ctypes.POINTER(f64)]
         L.dfsnufft_server_stats_get.argtypes = [vp, ctypes.POINTER(ServerStats)]
         L.dfsnufft_server_destroy.argtypes = [vp]
+        L.dfsnufft_plan_selftest_scan_timeout.argtypes = [vp, vp, vp, vp, ctypes.c_longlong]
         L.dfsnufft_set_points.argtypes = [vp, i64, vp, vp]
         L.dfsnufft_set_points_host.argtypes = [vp, i64, vp, vp]
         L.dfsnufft_execute.argtypes = [vp, vp, vp]
@@ -308,6 +310,14 @@ def dfsnufft_set_points_batch(h, counts, lon_ptr, colat_ptr):
     c = np.ascontiguousarray(counts, dtype=np.int64)
     _check(lib().dfsnufft_set_points_batch(h, c.ctypes.data, ctypes.c_void_p(lon_ptr),
                                            ctypes.c_void_p(colat_ptr)), h)
+
+
+def dfsnufft_plan_selftest_scan_timeout(h, counts, lon_ptr, colat_ptr, cycles):
+    """Status of a set_points whose bin scan waits in vain (ERR_TIMEOUT is the
+    expected outcome)."""
+    c = np.ascontiguousarray(counts, dtype=np.int64)
+    return lib().dfsnufft_plan_selftest_scan_timeout(h, c.ctypes.data, ctypes.c_void_p(lon_ptr),
+                                                     ctypes.c_void_p(colat_ptr), int(cycles))
 
 
 def dfsnufft_set_points(h, n_points, lon_ptr, colat_ptr):
