@@ -20,6 +20,10 @@ extern "C" {
  * Returns 0 and writes *flops_per_s, or a dfsnufft status code. */
 int dfsnufft_probe_fma_rate(int dtype, double target_ms, double *flops_per_s);
 
+/* Leading Horner steps that the FP64 interpolation at kernel width w takes in
+ * plain FP32 (host only): what a test of their rounding needs to know. */
+int dfsnufft_probe_plain_horner_steps(int w);
+
 /* Self-test of the bounded waits: one CTA initialises an mbarrier that
  * nothing ever arrives on and waits on it with the same bounded wait the TMA
  * kernels use, giving up after `cycles` SM clock cycles (1 <= cycles <= 4e9,

@@ -227,6 +227,16 @@ __host__ __device__ __forceinline__ int dfs_cstride(int nbins, int tile_y) {
     return dfs_rowcount_offset(nbins) + ((nbins * tile_y + 3) & ~3);
 }
 
+// First steps of a weight polynomial's chain (df_chain, interp.cu) that FP64 plans
+// take in plain FP32, without the coefficients' low parts.  Their error, evaluated
+// on the fitted coefficients of both oversampling factors, is at most 4.0e-16 of
+// the largest weight (w = 14, sigma 4; double-single itself rounds at 3.6e-15);
+// one step more would be 2.6e-14 (w = 14), 3.4e-15 (15), 1.1e-14 (16), one step at w =
+// 13 4.2e-15.
+__host__ __device__ constexpr int dfs_plain_horner_steps(int w) {
+    return w >= 16 ? 2 : w >= 14 ? 1 : 0;
+}
+
 // The sorted points (or, DFSNUFFT_KEEP_ORDER, the points in the caller's order)
 // as the interpolation reads them: base cell, offsets and the point's index.
 // One 16-byte record in FP32; in FP64 the packed base and index beside the two

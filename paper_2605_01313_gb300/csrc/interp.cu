@@ -200,13 +200,12 @@ template <int W> struct HornerDF {
 // One chain of a weight polynomial in u = s^2, coefficients k0, k0 - 2, .. k1 of
 // tap a, by compensated Horner's rule (Graillat, Langlois and Louvet): an FP32
 // recurrence whose product and sum errors, with the low parts of the
-// coefficients and of u, run through a second one.  The first TOP steps are
-// plain FP32: on |s| <= 1/2 what they add is smaller than the weight by 1e-8 and
-// more, and their rounding stays below 4e-16 of the largest weight (TOP from the
-// fitted coefficients of both oversampling factors: 2 for w >= 15, 1 for w >= 13).
+// coefficients and of u, run through a second one.  The first steps
+// (dfs_plain_horner_steps) are plain FP32: on |s| <= 1/2 what they add is smaller
+// than the weight by 1e-8 and more.
 template <int W>
 __device__ __forceinline__ df32 df_chain(const HornerDF<W> &h, int a, int k0, int k1, df32 u) {
-    constexpr int TOP = W >= 15 ? 2 : W >= 13 ? 1 : 0;
+    constexpr int TOP = dfs_plain_horner_steps(W);
     float e = h.hi[a][k0];
     float err = TOP ? 0.f : h.lo[a][k0];
 #pragma unroll

@@ -71,6 +71,8 @@ int probe(double target_ms, double *out) {
 
 }  // namespace
 
+extern "C" int dfsnufft_probe_plain_horner_steps(int w) { return dfs_plain_horner_steps(w); }
+
 extern "C" int dfsnufft_probe_fma_rate(int dtype, double target_ms, double *flops_per_s) {
     if (!flops_per_s || !(target_ms > 0)) return DFSNUFFT_ERR_INVALID_ARG;
     if (dtype == DFSNUFFT_F64) return probe<double>(target_ms, flops_per_s);

@@ -47,7 +47,7 @@ EXPORTS = (
     "dfsnufft_departure_points", "dfsnufft_rotate_to_arrival", "dfsnufft_lagrange_interp",
     "dfsnufft_plan_latitudes", "dfsnufft_plan_host_copy_bytes",
     "dfsnufft_ensemble_set_persistent", "dfsnufft_ensemble_selftest_queue_timeout",
-    "dfsnufft_plan_selftest_scan_timeout",
+    "dfsnufft_plan_selftest_scan_timeout", "dfsnufft_probe_plain_horner_steps",
 )
 REAL_FIELDS = 1
 KEEP_ORDER = 2
@@ -202,6 +202,7 @@ def lib():
         L.dfsnufft_plan_host_copy_bytes.argtypes = [vp, ctypes.POINTER(i64), ctypes.POINTER(i64),
                                                     ctypes.POINTER(i64)]
         L.dfsnufft_probe_fma_rate.argtypes = [i32, f64, ctypes.POINTER(f64)]
+        L.dfsnufft_probe_plain_horner_steps.argtypes = [i32]
         L.dfsnufft_selftest_wait_timeout.argtypes = [ctypes.c_longlong, ctypes.POINTER(i32),
                                                      ctypes.POINTER(f64)]
         L.dfsnufft_execute_noalloc.argtypes = [i32, i32, f64, i32, i32, i64, vp, vp, vp, vp, vp]
@@ -385,6 +386,10 @@ def dfsnufft_probe_fma_rate(dtype, target_ms=20.0) -> float:
     out = ctypes.c_double()
     _check(lib().dfsnufft_probe_fma_rate(_dtype_code(dtype), float(target_ms), ctypes.byref(out)))
     return out.value
+
+
+def dfsnufft_probe_plain_horner_steps(w) -> int:
+    return int(lib().dfsnufft_probe_plain_horner_steps(int(w)))
 
 
 def dfsnufft_selftest_wait_timeout(cycles):
