@@ -121,3 +121,17 @@ def test_pr_f64_scaled_inputs(torch_cuda):
     for f in range(2):
         assert np.array_equal(vals[f], base * s[f])
         assert oracle.rel_linf(vals[f][idx], ref * s[f]) <= 1e-11
+
+
+@pytest.mark.parametrize("n_lon,n_lat,M,N", [(12, 130, 5, 128), (12, 256, 5, 255), (10, 400, 4, 399),
+                                             (12, 512, 5, 511), (12, 1023, 5, 1022),
+                                             (6, 1500, 2, 1499)])
+def test_pr_f64_long_columns(torch_cuda, n_lon, n_lat, M, N):
+    """Fine columns of 1024, 2048 and 4096 rows (compile-time lengths) and of 8192."""
+    rng = np.random.default_rng(720 + n_lat)
+    prs = np.stack([synth.random_pr_spectrum(rng, M, N, 1.0) for _ in range(2)])
+    lon, colat = rng.uniform(-1.0, 7.0, 150), rng.uniform(-math.pi, 2 * math.pi, 150)
+    vals = run_pr(torch_cuda, prs, lon, colat, n_lon, n_lat, "f64")
+    for f in range(2):
+        ref = reference(prs[f], lon, colat, n_lon, n_lat)
+        assert oracle.rel_linf(vals[f], ref) <= 1e-11
