@@ -171,11 +171,10 @@ struct ScanParams {
 };
 
 // Layout of a member's count slice (cstride ints, zeroed before each
-// set_points): the scan's ticket and completion counters and its failure flag, the
-// bin-row flags (bytes), one 64-bit word a chunk, then the row counts.
+// set_points): the scan's ticket and completion counters, the bin-row flags
+// (bytes), one 64-bit word a chunk, then the row counts.
 __device__ __forceinline__ int *ws_ticket(int *slice) { return slice; }
 __device__ __forceinline__ int *ws_done(int *slice) { return slice + 1; }
-__device__ __forceinline__ int *ws_failed(int *slice) { return slice + 2; }
 __device__ __forceinline__ unsigned char *ws_rows(int *slice) {
     return reinterpret_cast<unsigned char *>(slice + 4);
 }
@@ -294,11 +293,12 @@ __device__ __forceinline__ unsigned long long chunk_word(int flag, int ne, int s
 // needed row range.
 //
 // The wait is bounded (DFS_WAIT_CYCLES, about a second).  A chunk that gives up
-// sets DFS_STATUS_TIMEOUT and the member's failure flag and tells the chunks after
-// it; its starts are sums of fewer counts, so the scatter stays inside the
-// member's slice, but the list and the records have gaps.  The last CTA then
-// leaves n_tasks = -1 and an empty row range, whatever the chunks stored: no pass
-// reads the list or the records, and the interpolation writes NaN.
+// sets DFS_STATUS_TIMEOUT, counts itself as failed in the upper half of the
+// completion counter and tells the chunks after it; its starts are sums of fewer
+// counts, so the scatter stays inside the member's slice, but the list and the
+// records have gaps.  The last CTA then leaves n_tasks = -1 and an empty row range,
+// whatever the chunks stored: no pass reads the list or the records, and the
+// interpolation writes NaN.
 //
 // Bound by latency: a chain of a ticket, the row counts, two block scans and the
 // words before it.  One kernel in place of a row prefix, chunk sums and a second
@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     dfs_grid_wait();
     __shared__ unsigned s_bits[(DFS_MAX_ROW_BLOCKS + 31) / 32];
     __shared__ int s_chunk, s_last, s_best, s_pre[2];
+    bool failed = false;                       // warp 0's
     const int member = blockIdx.y, tid = threadIdx.x;
     int *slice = count_all + (size_t)member * sp.cstride;
     int *start = start_all + (size_t)member * sp.bstride;
@@ -358,7 +359,6 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     block_scan2(c, c > 0, ps, pn, ts, tn);
     if (tid < 32) {
         int bs = 0, bn = 0;
-        bool failed = false;
         if (tid == 0 && !(sp.mute && chunk == 0))
             *(volatile unsigned long long *)&words[chunk] = chunk_word(chunk ? 1 : 2, tn, ts);
         const long long t0 = clock64();
@@ -380,10 +380,7 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
             if (through) break;
         }
         if (tid == 0) {
-            if (failed) {
-                if (status) atomicExch(status, DFS_STATUS_TIMEOUT);
-                atomicExch(ws_failed(slice), 1);
-            }
+            if (failed && status) atomicExch(status, DFS_STATUS_TIMEOUT);
             if (chunk)
                 *(volatile unsigned long long *)&words[chunk] =
                     chunk_word(failed ? 3 : 2, bn + tn, bs + ts);
@@ -408,12 +405,16 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     // publish the flags, then count this CTA done
     __threadfence();
     __syncthreads();
-    if (tid == 0) s_last = atomicAdd(ws_done(slice), 1) == sp.nch - 1;
+    if (tid == 0) {
+        const int add = failed ? 0x10001 : 1;              // at most 1024 chunks
+        const int done = atomicAdd(ws_done(slice), add) + add;
+        s_last = (done & 0xffff) == sp.nch ? done : 0;
+    }
     __syncthreads();
     if (!s_last) return;
     __threadfence();
     finish_rowrange(sp, rows, s_bits, &s_best, rowrange + member);
-    if (tid == 0 && __ldcg(ws_failed(slice))) {
+    if (tid == 0 && s_last > 0xffff) {
         n_tasks[member] = -1;
         rowrange[member] = make_int2(0, 0);
     }
