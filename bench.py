@@ -215,9 +215,18 @@ class ClockSampler:
                 "reasons": sorted(reasons), "samples": len(sm)}
 
 
+def launch_bytes(prm, n_fields, n_points, rows):
+    """Algorithmic HBM bytes per launch of each stage with the sorted points as they
+    are stored: base cell packed in one int, index and two offsets (16 bytes in
+    FP32, 24 in FP64), 4 less a point than stage_bytes counts."""
+    b = stage_bytes(prm, n_fields, n_points, rows)
+    return dict(b, set_points=b["set_points"] - 4 * n_points, interp=b["interp"] - 4 * n_points)
+
+
 def stage_bytes(prm, n_fields, n_points, rows):
     """Algorithmic HBM bytes per launch of each stage (one execute of all fields):
-    what each stage must read and write once.  A real-field plan reads the
+    what each stage must read and write once, a sorted point taken as two ints of
+    base cell, two offsets and an index.  A real-field plan reads the
     coefficient columns m >= 0 (plus the Nyquist column) and keeps N1/2 + 1
     theta-pass columns; the fine grid holds the real part only."""
     cs = 16 if prm["dtype"] == 0 else 8
@@ -570,7 +579,7 @@ def measure(args, name, wl, ws, rank, dev, serving, cpu_seconds=None):
     # ---- roofline of the dominant kernel
     pk, pk_kind = peaks()
     per_stage_ms = {k: (v[0] / v[1] if v[1] else None) for k, v in stage.items()}
-    sbytes = stage_bytes(prm, F, P, stats["rows_needed"])
+    sbytes = launch_bytes(prm, F, P, stats["rows_needed"])
     if pr_in:       # the theta pass reads the partial-regularity arrays instead
         cs = 16 if prm["dtype"] == 0 else 8
         N1, N2 = prm["N1"], prm["N2"]
@@ -907,7 +916,7 @@ def measure_ensemble(args, name, ws, rank, dev, cpu_seconds):
         prm = nufft.dfsnufft_plan_get_params(ens.plan_handle(gi))
         sp_launches.append(set_points_launches(prm, max(pts[gi][2])))
         st = nufft.dfsnufft_plan_point_stats(ens.plan_handle(gi))
-        step_bytes += sum(stage_bytes(prm, 3 * m, sum(pts[gi][2]), st["rows_needed"]).values())
+        step_bytes += sum(launch_bytes(prm, 3 * m, sum(pts[gi][2]), st["rows_needed"]).values())
     pk, pk_kind = peaks()
     achieved = step_bytes / (total_ms / args.steps * 1e-3) / 1e9
     if rank != 0:

@@ -70,3 +70,14 @@ def test_fft_flops(bench):
     import math
     assert bench.fft_flops(C3_F32, F, ROWS, "theta_pass") == 3 * 1025 * 5.0 * 4096 * 12
     assert bench.fft_flops(C3_F32, F, ROWS, "phi_pass") == 3 * ROWS * 5.0 * 2048 * math.log2(2048)
+
+
+def test_launch_bytes(bench):
+    # the sorted records as stored: 16 bytes in FP32, 24 in FP64
+    b = bench.launch_bytes(C3_F32, F, P, ROWS)
+    assert b["interp"] == 3 * (2096 * 4096 * 4 + P * 4) + P * 16 == 161_742_848
+    assert b["set_points"] == P * 20 + P * 20 + P * 16
+    b64 = bench.launch_bytes(C3_F64, F, P, ROWS)
+    assert b64["interp"] == 3 * (2096 * 4096 * 8 + P * 8) + P * 24
+    s = bench.stage_bytes(C3_F32, F, P, ROWS)
+    assert all(b[k] == s[k] for k in ("theta_pass", "phi_pass"))
