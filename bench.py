@@ -265,12 +265,11 @@ def interp_flops(prm, n_fields, n_points):
 
 
 def df32_interp_ops(prm, n_fields, n_points):
-    """FP32 arithmetic instructions (FADD, FMUL, FFMA: one each) of one FP64
-    interpolation launch in compensated double-single arithmetic, a fixed measure
-    of its work (the kernel, k_interp_fx, sums in fixed point and needs about a
-    third fewer instructions), counted from its operations: TwoSum 6, TwoProduct 2,
-    a double-single product 7 (with its fast renormalisation), sum 11, Horner step
-    15, Dot2 step (one compensated multiply-add) 12.  Per point: the
+    """FP32 arithmetic instructions (FADD, FMUL, FFMA: one each) that one FP64
+    interpolation takes in compensated double-single arithmetic, counted from its
+    operations (the kernel, k_interp_fx, sums in fixed point: fx_interp_ops).  TwoSum
+    6, TwoProduct 2, a double-single product 7 (with its fast renormalisation), sum
+    11, Horner step 15, Dot2 step (one compensated multiply-add) 12.  Per point: the
     x and y weights, each (w + 1) / 2 mirror pairs of an even and an odd Horner
     chain (w - 1 steps together), one product s o and the two sums, plus u = s^2
     for each axis; per point and field, w stencil rows of w Dot2 steps, each row
@@ -280,6 +279,24 @@ def df32_interp_ops(prm, n_fields, n_points):
     weights = pairs * ((w - 1) * 15 + 7 + 2 * 11) + 7
     rows = w * (12 * w + 3 + 12)
     return n_points * (2 * weights + n_fields * rows)
+
+
+def fx_interp_ops(prm, n_fields, n_points):
+    """Arithmetic instructions of the FP64 interpolation's weights and sums
+    (k_interp_fx), counted from its operations; staging, loads, addresses and idle
+    lanes come on top.  Per point and axis, (w + 1) / 2 mirror pairs of an even and
+    an odd compensated Horner chain: w - 1 steps together of 12 (product and its
+    error 2, TwoSum 6, joining the errors 2, error recurrence 2), the leading ones
+    of w >= 14 plain (1 each), a renormalisation (3) a chain, the product s o (7) and
+    the two sums (11 each), plus u = s^2 (7); per tap weight its split into integer
+    and fraction (10) and two scalings.  Per x weight also the sums' starts (3) and
+    the choice by parity (3).  Per point, field and stencil row: 4 a tap (wide product,
+    permutation, two FMAs) and 9 to join the row."""
+    w = prm["w"]
+    pairs = (w + 1) // 2
+    plain = 2 * (2 if w >= 16 else 1 if w >= 14 else 0)
+    axis = pairs * (12 * (w - 1 - plain) + plain + 2 * 3 + 7 + 2 * 11) + 7 + w * (10 + 2)
+    return n_points * (2 * axis + 6 * w + n_fields * w * (4 * w + 9))
 
 
 def fft_flops(prm, n_fields, rows, stage):
@@ -588,14 +605,15 @@ def measure(args, name, wl, ws, rank, dev, serving, cpu_seconds=None):
               key=lambda k: per_stage_ms[k] or 0.0)
     dom_ms = per_stage_ms[dom]
     if wl.dtype == "f64" and dom == "interp" and not (prm["flags"] & 2):
-        # FP64 plans interpolate on the FP32 and integer units: the stage's work as
-        # FP32 instructions (df32_interp_ops) against the FP32 pipe's instruction
-        # rate, measured live by the FMA probe (FLOP/s / 2)
+        # FP64 plans interpolate on the FP32 and integer units: the instructions of
+        # the weights and sums (fx_interp_ops) against the rate at which instructions
+        # issue, that of FP32 FMAs (one a cycle on each scheduler), measured live by
+        # the FMA probe (FLOP/s / 2)
         fma32 = nufft.dfsnufft_probe_fma_rate("f32", 20.0)
-        ops = df32_interp_ops(prm, F, P)
+        ops = fx_interp_ops(prm, F, P)
         achieved = ops / (dom_ms * 1e-3) / 1e12
         roof = {"kernel": dom, "bound": "alu", "achieved": achieved, "peak": fma32 / 2e12,
-                "unit": "T FP32-instructions/s", "frac": achieved / (fma32 / 2e12),
+                "unit": "T instructions/s", "frac": achieved / (fma32 / 2e12),
                 "ops_per_launch": ops,
                 "peak_source": "measured FP32 FMA rate / 2 (dfsnufft_probe_fma_rate, "
                                "one FFMA instruction = 2 FLOP)",

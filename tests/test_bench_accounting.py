@@ -81,3 +81,16 @@ def test_launch_bytes(bench):
     assert b64["interp"] == 3 * (2096 * 4096 * 8 + P * 8) + P * 24
     s = bench.stage_bytes(C3_F32, F, P, ROWS)
     assert all(b[k] == s[k] for k in ("theta_pass", "phi_pass"))
+
+
+def test_fx_interp_ops(bench):
+    # w = 14: 7 pairs of chains with 13 steps together, 11 of them of 12 instructions
+    # and 2 plain, two renormalisations, a product and two sums: 169 a pair, u = s^2
+    # and 14 weights of 12 an axis; 6 more an x weight; per field 14 rows of 14 taps
+    axis = 7 * (11 * 12 + 2 + 2 * 3 + 7 + 2 * 11) + 7 + 14 * 12
+    assert axis == 1358
+    assert bench.fx_interp_ops(C3_F64, F, P) == P * (2 * axis + 84 + 3 * 14 * (14 * 4 + 9))
+    # no plain steps at w = 13, three fields of 13 rows
+    w13 = 7 * (12 * 12 + 6 + 7 + 22) + 7 + 13 * 12
+    assert bench.fx_interp_ops(dict(C3_F64, w=13), F, P) == \
+        P * (2 * w13 + 78 + 3 * 13 * (13 * 4 + 9))
