@@ -36,6 +36,9 @@
  *  - Streams: every device call is enqueued on the plan's CUDA stream and
  *    returns after enqueue (asynchronous); results are ready when the stream
  *    reaches that point.  A plan is not thread-safe.
+ *  - Alignment: device pointers are multiples of their element's size (8 bytes for
+ *    points; 8 or 16 for complex and 4 or 8 for real values of F32 or F64 plans);
+ *    others are refused with DFSNUFFT_ERR_INVALID_ARG.
  *  - Ownership: the caller allocates and owns every input and output buffer.
  *    The plan owns its fine grids, deconvolution factors, twiddle tables and
  *    sorted point data; set_points copies what it needs, so the point

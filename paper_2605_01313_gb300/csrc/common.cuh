@@ -290,6 +290,19 @@ __host__ __forceinline__ DfsPoints<double> dfs_points<double>(const dfsnufft_pla
     return DfsPoints<double>{(int2 *)p->d_base, (double2 *)p->d_frac};
 }
 
+// The kernels read and write whole elements, reals and complex values of twice
+// their size: a device pointer off its element's size would fault, so the entry
+// points refuse it.
+__host__ __forceinline__ bool dfs_aligned(const void *ptr, size_t bytes) {
+    return (reinterpret_cast<uintptr_t>(ptr) & (bytes - 1)) == 0;
+}
+__host__ __forceinline__ bool dfs_real_aligned(const dfsnufft_plan_s *p, const void *ptr) {
+    return dfs_aligned(ptr, p->prm.dtype == DFSNUFFT_F64 ? sizeof(double) : sizeof(float));
+}
+__host__ __forceinline__ bool dfs_complex_aligned(const dfsnufft_plan_s *p, const void *ptr) {
+    return dfs_aligned(ptr, p->prm.dtype == DFSNUFFT_F64 ? sizeof(double2) : sizeof(float2));
+}
+
 // The line window of the next launches: first line and count.
 __host__ __forceinline__ void dfs_lines(const dfsnufft_plan_s *p, int &line0, int &nlines) {
     line0 = p->nwin ? p->win0 : 0;

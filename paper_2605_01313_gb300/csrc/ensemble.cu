@@ -165,7 +165,10 @@ extern "C" int dfsnufft_ensemble_run(dfsnufft_ensemble e, const int64_t *const *
     std::vector<const void *> ptr;
     std::vector<int64_t> counts;
     for (int g = 0; g < e->n_groups; ++g) {
-        if (!n_points[g] || !lon[g] || !colat[g] || !coeffs[g] || !values[g])
+        if (!n_points[g] || !lon[g] || !colat[g] || !coeffs[g] || !values[g] ||
+            !dfs_aligned(lon[g], sizeof(double)) || !dfs_aligned(colat[g], sizeof(double)) ||
+            !dfs_complex_aligned(e->plans[g], coeffs[g]) ||
+            !dfs_real_aligned(e->plans[g], values[g]))
             return DFSNUFFT_ERR_INVALID_ARG;
         ptr.push_back(lon[g]);
         ptr.push_back(colat[g]);

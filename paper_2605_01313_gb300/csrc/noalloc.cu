@@ -82,6 +82,10 @@ extern "C" int dfsnufft_execute_noalloc(int n_lon, int n_lat, double tol, int dt
     if (n_fields < 1 || n_fields > 64 || n_points < 1 || n_points > 0x7fffffffLL || !lon ||
         !colat || !coeffs || !values)
         return DFSNUFFT_ERR_INVALID_ARG;
+    const size_t element = dtype == DFSNUFFT_F64 ? sizeof(double) : sizeof(float);
+    if (!dfs_aligned(lon, sizeof(double)) || !dfs_aligned(colat, sizeof(double)) ||
+        !dfs_aligned(coeffs, 2 * element) || !dfs_aligned(values, element))
+        return DFSNUFFT_ERR_INVALID_ARG;
     dfsnufft_params prm;
     int rc = dfsnufft_choose_params(n_lon, n_lat, tol, dtype, &prm);
     if (rc != DFSNUFFT_OK) return rc;

@@ -745,7 +745,9 @@ extern "C" int dfsnufft_set_points_batch(dfsnufft_plan p, const int64_t *n_point
                                          const double *lon, const double *colat) {
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
     if (p->status) return p->status;
-    if (!n_points || !lon || !colat) return DFSNUFFT_ERR_INVALID_ARG;
+    if (!n_points || !lon || !colat || !dfs_aligned(lon, sizeof(double)) ||
+        !dfs_aligned(colat, sizeof(double)))
+        return DFSNUFFT_ERR_INVALID_ARG;
     int rc = update_counts(p, n_points);
     if (rc) return rc;
     p->has_points = 0;
@@ -785,7 +787,8 @@ extern "C" int dfsnufft_execute(dfsnufft_plan p, const void *coeffs, void *value
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
     if (p->status) return p->status;
     if (!p->has_points) return DFSNUFFT_ERR_NO_POINTS;
-    if (!coeffs || !values) return DFSNUFFT_ERR_INVALID_ARG;
+    if (!coeffs || !values || !dfs_complex_aligned(p, coeffs) || !dfs_real_aligned(p, values))
+        return DFSNUFFT_ERR_INVALID_ARG;
     DFS_CK(p, timing_begin(p, 1));
     DFS_CK(p, dfs_launch_theta_pass(p, coeffs));
     DFS_CK(p, timing_end(p, 1));
@@ -802,7 +805,8 @@ extern "C" int dfsnufft_execute_pr(dfsnufft_plan p, int M, int N, const void *pr
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
     if (p->status) return p->status;
     if (!p->has_points) return DFSNUFFT_ERR_NO_POINTS;
-    if (!pr || !values || !p->herm) return DFSNUFFT_ERR_INVALID_ARG;
+    if (!pr || !values || !p->herm || !dfs_complex_aligned(p, pr) || !dfs_real_aligned(p, values))
+        return DFSNUFFT_ERR_INVALID_ARG;
     if (M < 0 || M > p->prm.N1 / 2 - 1 || N < 1 || N > p->prm.N2 / 2 - 1)
         return DFSNUFFT_ERR_INVALID_ARG;
     DFS_CK(p, timing_begin(p, 1));
@@ -841,7 +845,9 @@ static int grid_to_coeffs(dfsnufft_plan p, const void *samples, const int *parit
                           void *coeffs, bool full) {
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
     if (p->status) return p->status;
-    if (!samples || !parity || !coeffs) return DFSNUFFT_ERR_INVALID_ARG;
+    if (!samples || !parity || !coeffs || !dfs_real_aligned(p, samples) ||
+        !dfs_complex_aligned(p, coeffs))
+        return DFSNUFFT_ERR_INVALID_ARG;
     if (!dfs_forward_supported(p->prm)) return DFSNUFFT_ERR_UNSUPPORTED;
     int rc = set_parity(p, parity);
     if (rc) return rc;
@@ -867,7 +873,9 @@ extern "C" int dfsnufft_interpolate_grid(dfsnufft_plan p, const void *samples, c
     if (!p) return DFSNUFFT_ERR_INVALID_ARG;
     if (p->status) return p->status;
     if (!p->has_points) return DFSNUFFT_ERR_NO_POINTS;
-    if (!samples || !parity || !values) return DFSNUFFT_ERR_INVALID_ARG;
+    if (!samples || !parity || !values || !dfs_real_aligned(p, samples) ||
+        !dfs_real_aligned(p, values))
+        return DFSNUFFT_ERR_INVALID_ARG;
     if (!dfs_forward_supported(p->prm)) return DFSNUFFT_ERR_UNSUPPORTED;
     if (!p->d_coef_stage) {
         const size_t cs = p->prm.dtype == DFSNUFFT_F64 ? sizeof(double2) : sizeof(float2);
