@@ -144,9 +144,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
 // Per precision: elements per thread E, threads per CTA at most MAXT with MINB
 // resident CTAs (MINBH for the rows of real-field plans); rows longer than
 // E x MAXT complex values (FP32 fine grids of 8192 columns) use the wide form of
-// MAXTW threads.  Double-single rows of real-field plans fit 64 registers a
-// thread without spills, so two CTAs share an SM (C3 FP64 phi pass 305 -> 256
-// us); the general rows would spill there and keep one.
+// MAXTW threads.  Double-single rows of real-field plans run with 64
+// registers a thread, so that two CTAs share an SM (2048 x 1024 in FP64: 305 -> 256
+// us): at most 8 bytes of spills at the compile-time lengths, 64 at the run-time
+// one.  The general rows keep one CTA (117 registers; 40 bytes at the run-time
+// length).
 template <typename R> struct PhiCfg;
 template <> struct PhiCfg<float> {
     static const int E = DFS_FFT_E, MAXT = 256, MINB = 3, MINBH = 3, MAXTW = 512;

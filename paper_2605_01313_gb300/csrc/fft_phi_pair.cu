@@ -10,7 +10,7 @@
 // eight inputs straight from the theta pass's output, all in flight at once and
 // each value twice (the second read hits the L1 cache): no staging pass over
 // shared memory and no barrier before the transform.  Bound by the shared-memory
-// and global-access wavefronts (68% of the L1 data pipe at 2048 x 1024).
+// and global-access wavefronts (79% of the L1 data pipe at 2048 x 1024).
 // Measured against the staged, scalar form: three lines of 2080 rows x 4096
 // cells 58 -> 40 us, of 4112 x 8192 (run-time length before) 488 -> 165 us, 48
 // lines of 2048 cells 212 -> 139 us.

@@ -26,8 +26,10 @@
 // e^{2 pi i n s / n2} e^{2 pi i n q / (n2/2)}, s = 0, 1 (the modes fit in n2/2;
 // when n2 = 2 N2 the two Nyquist modes n = -N2/2 and n = +N2/2 of a real-field
 // plan share index N2/2 and are added there).  k_theta_pass is the plain-load
-// version: FP64 plans' partial-regularity input, and the shapes the others
-// (FP64 plans in double-single arithmetic: fft_theta_df.cu) do not take (unaligned coefficient pointer, CTA or shared-memory limits).
+// version: partial-regularity input of FP64 plans, the allocation-free call, and
+// what the others (FP64 plans in double-single arithmetic: fft_theta_df.cu) do not
+// take: FP32 coefficients or a first column 8 bytes off a 16-byte boundary (odd
+// N1/2 of a real-field plan), fine columns shorter or longer than theirs.
 #include <type_traits>
 
 #include "coef_map.cuh"
@@ -85,7 +87,11 @@ struct ThetaArgs {
 // grid (ceil(tcols / CB), lines); block CB * n2/E threads, thread = (t, c) with c fastest.
 // PRIN (real-field plans): the input is partial-regularity DFS coefficients,
 // lines x (prM + 1) x (prN + 1) complex, converted on the fly by pr_coef.
-// LOGN > 0: length n2 = 2^LOGN at compile time with the stage-ordered table stw.
+// LOGN > 0: length n2 = 2^LOGN at compile time with the stage-ordered table stw
+// (partial-regularity input of FP64 plans).
+// T of FP32 plans is stored by row pairs (t_store), which costs this kernel two
+// 4-byte stores a value: 131 -> 133 us on unaligned coefficients of 2048 x 1024,
+// 32.7 on those of 1024 x 512 either way; the phi pass of the pairs wins 18 and 6 us.
 // emax (double-single passes): each line's largest coefficient exponent, from
 // k_coef_maxexp; the line is transformed at the scale of df_line_shift.
 template <typename R, int E, int MAXT, int MINB, bool HERM, bool PRIN = false,
@@ -328,7 +334,7 @@ __global__ void __launch_bounds__(MAXT, MINB)
 }
 
 // Per precision: elements per thread E, threads per CTA at most MAXT, resident
-// CTAs MINB the register budget is set for (plain kernel); for the TMA kernel
+// CTAs MINB the register budget is set for (plain kernel); for the TMA kernel (FP64)
 // columns per block CB, threads at most TMAXT and TMINB resident CTAs per SM.
 template <typename R> struct ThetaCfg;
 template <> struct ThetaCfg<float> {
@@ -339,7 +345,7 @@ template <> struct ThetaCfg<double> {
 };
 // Double-single: two CTAs of one column each per SM.
 template <> struct ThetaCfg<df32> {
-    static const int E = DFS_FFT_E, MAXT = 512, MINB = 2, CB = 1, TMAXT = 512, TMINB = 1;
+    static const int E = DFS_FFT_E, MAXT = 512, MINB = 2;
 };
 
 template <typename R, int CB, int LOGH, bool HERM, bool PRIN>
