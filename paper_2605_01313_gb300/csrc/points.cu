@@ -166,8 +166,7 @@ struct ScanParams {
     int cstride;              // per-member stride of the count slice (scan workspace + counts)
     int nch;                  // chunks of DFS_SCAN_CHUNK bins
     int tile_y, c0, w, n2;
-    long long budget;         // SM cycles the look-back waits at most
-    int mute;                 // self-test: chunk 0 publishes nothing
+    long long budget;         // SM cycles the look-back waits at most (self-test)
 };
 
 // Layout of a member's count slice (cstride ints, zeroed before each
@@ -298,12 +297,15 @@ __device__ __forceinline__ unsigned long long chunk_word(int flag, int ne, int s
 // counts, so the scatter stays inside the member's slice, but the list and the
 // records have gaps.  The last CTA then leaves n_tasks = -1 and an empty row range,
 // whatever the chunks stored: no pass reads the list or the records, and the
-// interpolation writes NaN.
+// interpolation writes NaN.  SELFTEST: the same with a limit of the caller's, and
+// chunk 0 publishes nothing, so that every other chunk gives up (a form of its own,
+// since both as kernel parameters cost 1 us of the 42 of set_points).
 //
 // Bound by latency: a chain of a ticket, the row counts, two block scans and the
 // words before it.  One kernel in place of a row prefix, chunk sums and a second
 // scan pass whose last CTA searched the row gaps serially: 17 us in three
 // launches -> 9.8 us (32768 bins), 13 -> 8 us (2048 bins).
+template <bool SELFTEST>
 __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
                                                          int *__restrict__ count_all,
                                                          int *__restrict__ start_all,
@@ -359,8 +361,9 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
     block_scan2(c, c > 0, ps, pn, ts, tn);
     if (tid < 32) {
         int bs = 0, bn = 0;
-        if (tid == 0 && !(sp.mute && chunk == 0))
+        if (tid == 0 && !(SELFTEST && chunk == 0))
             *(volatile unsigned long long *)&words[chunk] = chunk_word(chunk ? 1 : 2, tn, ts);
+        const long long budget = SELFTEST ? sp.budget : DFS_WAIT_CYCLES;
         const long long t0 = clock64();
         for (int base = chunk - 1; base >= 0; base -= 32) {
             const int idx = base - tid;
@@ -368,7 +371,7 @@ __global__ void __launch_bounds__(DFS_SCAN_CHUNK) k_scan(ScanParams sp,
             bool late = false;
             if (idx >= 0) {
                 volatile unsigned long long *p = &words[idx];
-                while (((w = *p) >> 62) == 0 && !late) late = clock64() - t0 > sp.budget;
+                while (((w = *p) >> 62) == 0 && !late) late = clock64() - t0 > budget;
                 late |= (w >> 62) == 3;
             }
             failed = __any_sync(0xffffffffu, late);
@@ -614,8 +617,7 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
     sp.c0 = p->c0;
     sp.w = q.w;
     sp.n2 = q.n2;
-    sp.budget = p->scan_budget ? p->scan_budget : DFS_WAIT_CYCLES;
-    sp.mute = p->scan_budget != 0;
+    sp.budget = p->scan_budget;
     if (!p->keep_order && p->max_member_points <= SMALL_POINTS &&
         p->nbins * q.tile_y <= SMALL_KEYS)
         return q.dtype == DFSNUFFT_F64 ? launch_points_small<double>(p, lon, colat, f, sp)
@@ -644,9 +646,10 @@ cudaError_t dfs_launch_set_points(dfsnufft_plan p, const double *lon, const doub
                                                          rowoff, p->d_bin_count,
                                                          (FoldRec<float> *)p->d_urec);
     // the kernels after the fold start launching while their predecessor drains
-    if ((e = dfs_launch_dependent(k_scan, dim3(p->nch, M), dim3(DFS_SCAN_CHUNK), 0, p->stream, sp,
-                                  p->d_bin_count, p->d_bin_start, p->d_task_bin, p->d_n_tasks,
-                                  p->d_rowrange, p->d_status)))
+    if ((e = dfs_launch_dependent(sp.budget ? k_scan<true> : k_scan<false>, dim3(p->nch, M),
+                                  dim3(DFS_SCAN_CHUNK), 0, p->stream, sp, p->d_bin_count,
+                                  p->d_bin_start, p->d_task_bin, p->d_n_tasks, p->d_rowrange,
+                                  p->d_status)))
         return e;
     if (q.dtype == DFSNUFFT_F64)
         return dfs_launch_dependent(k_scatter<double>, grid, dim3(tpb), 0, p->stream,
