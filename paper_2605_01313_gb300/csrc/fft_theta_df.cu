@@ -10,7 +10,7 @@
 // the modes in its first and last quarter: the first radix-8 stage adds nothing
 // to the zeros between.
 //
-// Bound by FP32 instructions and the exchanges (54% of the issue slots).  2048 x
+// Bound by FP32 instructions and the exchanges (49% of the issue slots).  2048 x
 // 1024, three fields: an exponent pass of 40 us and a plain-load theta pass of 388
 // us (16-byte strided loads) before, 344 us in this form with the butterflies'
 // earlier arithmetic; 64 x 32: 39 us in two launches (two CTAs of 512 threads) to

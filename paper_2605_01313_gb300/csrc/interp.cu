@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a, const __grid_const
 // over the FMA pipes and the ALU, where a compensated floating-point step (Dot2)
 // takes 12 instructions and a product of two-limb integers three wide products.
 // 2.1M points, three fields, w = 14: 1122 us with Dot2, 836 with two-limb
-// integers, 726 in this form (65% of the issue slots; more warps an SM, narrower
+// integers, 726 in this form (64% of the issue slots; more warps an SM, narrower
 // bins and the fields' sums interleaved were no faster).  Of its 8600
 // instructions per 32 points the weights take a third and the tiles' staging a
 // twelfth.
