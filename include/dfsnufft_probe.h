@@ -13,6 +13,9 @@
 extern "C" {
 #endif
 
+struct dfsnufft_plan_s;
+struct dfsnufft_ensemble_s;
+
 /* Measure the device's fused multiply-add rate in FLOP/s (2 per FMA) for
  * dtype DFSNUFFT_F64 (0) or DFSNUFFT_F32 (1): a kernel of independent FMA
  * chains, one CTA per SM slot, timed with CUDA events on the legacy default
